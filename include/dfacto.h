@@ -388,7 +388,7 @@ dfacto_status dfacto_joint_objective(dfacto_t* h, double* obj_out);
  * once.  Jobs that share (R, factor type) form a rank class: their flattened
  * CSR copies are concatenated into one block-diagonal tensor (indices offset
  * per job) and their factors are pooled, so the MTTKRP of a mode for every
- * job of every class is one persistent kernel launch.  The per-job steps
+ * job of a class is one kernel launch.  The per-job steps
  * (Gamma^{-1}, N Gamma^{-1}, normalisation, Grams, fit) run as one batched
  * launch per step and rank class, and from the second sweep on the whole
  * sweep is replayed as one CUDA graph.

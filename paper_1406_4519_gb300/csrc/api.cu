@@ -251,7 +251,7 @@ void dfacto_destroy(dfacto_t* h) {
   for (int m = 0; m < 3; ++m) {
     ModeCSR& M = h->m[m];
     for (void* q : {(void*)M.fiber_ptr, (void*)M.fiber_idx, (void*)M.fiber_row, (void*)M.nz_ptr,
-                    (void*)M.nz_idx, (void*)M.nz_val, (void*)M.end_bits, (void*)M.seg_fib,
+                    (void*)M.nz_idx, (void*)M.nz_val, (void*)M.end_bits, (void*)M.row_bits, (void*)M.seg_fib,
                     h->F[m], (void*)h->grad[m], (void*)h->gram[m]})
       if (q) cudaFreeAsync(q, h->stream);
   }
@@ -382,7 +382,10 @@ dfacto_status dfacto_build(const int32_t* idx, const float* val, int64_t nnz, co
     return st;
   }
   for (int m = 0; m < 3; ++m) {
-    h->m[m].cfg = choose_walk(R, h->dtype, nnz, h->m[m].nfib, opt.seg_nnz, opt.vec);
+    // the walk's own rank and gathered type (padded FP32 copies at a padded rank)
+    const int RP = walk_rank(R, opt.vec);
+    h->m[m].cfg = RP != R ? choose_walk(RP, DFACTO_F32, nnz, h->m[m].nfib, opt.seg_nnz, 0)
+                          : choose_walk(R, h->dtype, nnz, h->m[m].nfib, opt.seg_nnz, opt.vec);
     if (opt.walk > 0) {
       h->m[m].cfg.kernel = opt.walk;
     }
@@ -398,13 +401,10 @@ dfacto_status dfacto_get_info(dfacto_t* h, dfacto_info* info) {
   std::memcpy(info->dims, h->dims, sizeof(h->dims));
   info->rank = h->R;
   info->nnz = h->nnz;
-  const int RP = walk_rank(h->R, h->opt.vec);
   for (int m = 0; m < 3; ++m) {
     info->nfib[m] = h->m[m].nfib;
     info->seg_nnz[m] = h->m[m].cfg.seg;
-    info->vec[m] = (RP != h->R)
-                       ? choose_walk(RP, DFACTO_F32, h->nnz, h->m[m].nfib, h->opt.seg_nnz, 0).vec
-                       : h->m[m].cfg.vec;
+    info->vec[m] = h->m[m].cfg.vec;
   }
   info->device_bytes = h->bytes;
   info->factor_dtype = h->dtype;

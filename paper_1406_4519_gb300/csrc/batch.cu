@@ -7,8 +7,8 @@
 // jobs' dimensions), and the factors of each mode sit in one pool in the same
 // order.  The MTTKRP of Algorithm 1 over the class is then exactly the
 // MTTKRPs of its jobs stacked: a nonzero of job j only ever reads rows of job
-// j's factors and writes rows of job j's output.  The walk of every class of
-// one factor type runs in one persistent launch (mttkrp_walk2_multi).
+// j's factors and writes rows of job j's output, so a class is one walk
+// (mttkrp_walk2).
 //
 // The R x R and row steps of Algorithm 2 run once per rank class as batched
 // launches (each block finds its job and runs that job's step); from the
@@ -82,6 +82,7 @@ struct ClassMode {
   int32_t* nz_idx = nullptr;     // [nnz]
   float* nz_val = nullptr;       // [nnz]
   uint32_t* end_bits = nullptr;  // [(nnz + 31) / 32]
+  uint32_t* row_bits = nullptr;  // [(nnz + 31) / 32]
   int32_t* seg_fib = nullptr;    // [nseg_cap]
   float* N = nullptr;            // [dim_o x R] MTTKRP output of every job of the class
 };
@@ -96,7 +97,6 @@ struct BatchClass {
   void* F[3] = {nullptr, nullptr, nullptr};  // factor pools [rows[m] x R]
   ClassMode m[3];
   WalkCfg cfg;
-  int shape = -1;                  // multi shape id (-1: own launch)
   int64_t nseg_cap = 0;            // seg_fib capacity (segments)
   float* carry = nullptr;          // [carry_cap x 2 x R]
   int32_t* carry_row = nullptr;    // [carry_cap x 2]
@@ -119,7 +119,6 @@ struct BatchClass {
 
 struct dfacto_batch {
   int device = 0;
-  int sms = 152;
   std::vector<dfacto_t*> jobs;
   std::vector<dfacto::BatchClass> cls;
   cudaStream_t user = nullptr;   // the caller's stream
@@ -197,12 +196,19 @@ dfacto_status build_class_mode(dfacto_batch* b, BatchClass& C, int mode) {
   if (M.nfib >= (int64_t(1) << 31)) return bfail(b, DFACTO_EINVAL, "rank class has 2^31 fibers or more");
   dfacto_status st;
   if ((st = balloc(b, &M.fiber_ptr, sizeof(int64_t) * (size_t)(M.dim_o + 1))) != DFACTO_OK) return st;
-  if ((st = balloc(b, &M.fiber_idx, sizeof(int32_t) * (size_t)M.nfib)) != DFACTO_OK) return st;
+  if ((st = balloc(b, &M.fiber_idx, sizeof(int32_t) * (size_t)(M.nfib + 1))) != DFACTO_OK) return st;
   if ((st = balloc(b, &M.fiber_row, sizeof(int32_t) * (size_t)M.nfib)) != DFACTO_OK) return st;
+  DB_CUDA(b, cudaMemsetAsync(M.fiber_idx + M.nfib, 0, sizeof(int32_t), s));
   if ((st = balloc(b, &M.nz_ptr, sizeof(int64_t) * (size_t)(M.nfib + 1))) != DFACTO_OK) return st;
-  if ((st = balloc(b, &M.nz_idx, sizeof(int32_t) * (size_t)C.nnz)) != DFACTO_OK) return st;
-  if ((st = balloc(b, &M.nz_val, sizeof(float) * (size_t)C.nnz)) != DFACTO_OK) return st;
-  if ((st = balloc(b, &M.end_bits, sizeof(uint32_t) * (size_t)((C.nnz + 31) / 32))) != DFACTO_OK) return st;
+  const size_t npad = (size_t)walk_padded(C.nnz);
+  if ((st = balloc(b, &M.nz_idx, sizeof(int32_t) * npad)) != DFACTO_OK) return st;
+  if ((st = balloc(b, &M.nz_val, sizeof(float) * npad)) != DFACTO_OK) return st;
+  if ((st = balloc(b, &M.end_bits, sizeof(uint32_t) * (npad / 32))) != DFACTO_OK) return st;
+  if ((st = balloc(b, &M.row_bits, sizeof(uint32_t) * (npad / 32))) != DFACTO_OK) return st;
+  if (npad > (size_t)C.nnz) {
+    DB_CUDA(b, cudaMemsetAsync(M.nz_idx + C.nnz, 0, sizeof(int32_t) * (npad - (size_t)C.nnz), s));
+    DB_CUDA(b, cudaMemsetAsync(M.nz_val + C.nnz, 0, sizeof(float) * (npad - (size_t)C.nnz), s));
+  }
   if ((st = balloc(b, &M.N, sizeof(float) * (size_t)M.dim_o * C.R)) != DFACTO_OK) return st;
   for (size_t t = 0; t < C.jobs.size(); ++t) {
     const dfacto_t* h = b->jobs[C.jobs[t]];
@@ -233,7 +239,7 @@ dfacto_status build_class_mode(dfacto_batch* b, BatchClass& C, int mode) {
   set_i64<<<1, 1, 0, s>>>(M.nz_ptr + M.nfib, C.nnz);
   DF_COUNT();
   DB_CUDA(b, cudaGetLastError());
-  DB_CUDA(b, launch_fiber_end_bits(M.nz_ptr, M.nfib, C.nnz, M.end_bits, s));
+  DB_CUDA(b, launch_walk_bits(M.nz_ptr, M.fiber_row, M.nfib, C.nnz, M.end_bits, M.row_bits, s));
   return DFACTO_OK;
 }
 
@@ -260,6 +266,7 @@ MttkrpParams class_params(const BatchClass& C, int mode, int32_t* bad) {
   a.nz_val = M.nz_val;
   a.seg_fib = M.seg_fib;
   a.end_bits = M.end_bits;
+  a.row_bits = M.row_bits;
   a.Fin = C.F[(mode + 1) % 3];
   a.Ff = C.F[(mode + 2) % 3];
   a.out = M.N;
@@ -273,54 +280,23 @@ MttkrpParams class_params(const BatchClass& C, int mode, int32_t* bad) {
   return a;
 }
 
-// MTTKRP of `mode` for the classes in `which` (all classes if empty): the
-// classes with a compiled multi shape share one persistent launch per factor
-// type (kMaxClasses at a time), the others get their own walk; then one
-// fix-up per class.
+// MTTKRP of `mode` for the classes in `which` (all classes if empty): one walk
+// and one fix-up per class.  (A persistent kernel holding every class's walk
+// shape needs the registers of the widest one and spills; a class's own kernel
+// does not, and the classes are large enough that its last wave costs little.)
 dfacto_status batch_mttkrp_issue(dfacto_batch* b, int mode, cudaStream_t s,
                                  const std::vector<int>& which) {
   std::vector<int> ks = which;
   if (ks.empty())
     for (int k = 0; k < (int)b->cls.size(); ++k) ks.push_back(k);
-  for (int dtype : {DFACTO_F32, DFACTO_BF16}) {
-    std::vector<int> multi;
-    for (int k : ks) {
-      const BatchClass& C = b->cls[k];
-      if (C.dtype != dtype || C.nnz == 0) continue;
-      if (C.shape >= 0) {
-        multi.push_back(k);
-      } else {
-        const MttkrpParams a = class_params(C, mode, b->d_bad);
-        cudaError_t e = dtype == DFACTO_BF16
-                            ? launch_walk2<__nv_bfloat16>(C.cfg.vec, C.cfg.G, a, C.ncta(), s)
-                            : launch_walk2<float>(C.cfg.vec, C.cfg.G, a, C.ncta(), s);
-        if (e != cudaSuccess) return bcuda(b, e, "batched walk (own launch)");
-      }
-    }
-    for (size_t i0 = 0; i0 < multi.size(); i0 += kMaxClasses) {
-      MultiWalkParams mp;
-      std::memset(&mp, 0, sizeof(mp));
-      size_t smem = 0;
-      int total = 0;
-      mp.nclass = (int)std::min<size_t>(kMaxClasses, multi.size() - i0);
-      for (int c = 0; c < mp.nclass; ++c) {
-        const BatchClass& C = b->cls[multi[i0 + c]];
-        mp.p[c] = class_params(C, mode, b->d_bad);
-        mp.shape[c] = C.shape;
-        mp.cta_begin[c] = total;
-        total += (int)C.ncta();
-        smem = std::max(smem, walk2_smem_bytes(C.cfg.vec, C.cfg.G, C.R));
-      }
-      mp.cta_begin[mp.nclass] = total;
-      for (int c = mp.nclass + 1; c <= kMaxClasses; ++c) mp.cta_begin[c] = total;
-      // Persistent grid: as many blocks as stay resident (3 per SM at 80
-      // registers, fewer if shared memory limits them).
-      const int per_sm = std::max<int>(1, std::min<int>(3, (int)((228 * 1024) / (smem + 2048 + 1024))));
-      const int grid = std::min(total, b->sms * per_sm);
-      cudaError_t e = dtype == DFACTO_BF16 ? launch_walk2_multi<__nv_bfloat16>(mp, smem, grid, s)
-                                           : launch_walk2_multi<float>(mp, smem, grid, s);
-      if (e != cudaSuccess) return bcuda(b, e, "batched walk");
-    }
+  for (int k : ks) {
+    const BatchClass& C = b->cls[k];
+    if (C.nnz == 0) continue;
+    const MttkrpParams a = class_params(C, mode, b->d_bad);
+    cudaError_t e = C.dtype == DFACTO_BF16
+                        ? launch_walk2<__nv_bfloat16>(C.cfg.vec, C.cfg.G, a, C.ncta(), s)
+                        : launch_walk2<float>(C.cfg.vec, C.cfg.G, a, C.ncta(), s);
+    if (e != cudaSuccess) return bcuda(b, e, "batched walk");
   }
   for (int k : ks) {
     const BatchClass& C = b->cls[k];
@@ -363,7 +339,7 @@ std::vector<WalkCfg> candidates(const BatchClass& C) {
   for (int vec : {4, 8}) {
     if (C.R % vec != 0) continue;
     const int G = next_pow2((C.R + vec - 1) / vec);
-    if (G > 32 || multi_shape_id(vec, G) < 0) continue;
+    if (G > 32 || (vec == 8 && G > 16)) continue;
     for (int seg : kTuneSegs) {
       WalkCfg c;
       c.vec = vec;
@@ -384,7 +360,6 @@ dfacto_status autotune_class(dfacto_batch* b, int k) {
   double best_ms = 1e300;
   for (const WalkCfg& c : cands) {
     C.cfg = c;
-    C.shape = multi_shape_id(c.vec, c.G);
     dfacto_status st = prepare_walk(b, C);
     if (st != DFACTO_OK) return st;
     double ms = 0;
@@ -395,7 +370,6 @@ dfacto_status autotune_class(dfacto_batch* b, int k) {
     }
   }
   C.cfg = best;
-  C.shape = multi_shape_id(best.vec, best.G);
   C.tuned_ms = best_ms;
   return prepare_walk(b, C);
 }
@@ -614,7 +588,6 @@ dfacto_status dfacto_batch_create(dfacto_t* const* jobs, int32_t n, const dfacto
   b->opt = opt;
   b->user = static_cast<cudaStream_t>(stream);
   b->jobs.assign(jobs, jobs + n);
-  cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
   auto bail = [&](dfacto_status st) {
     release(b);
     delete b;
@@ -668,7 +641,6 @@ dfacto_status dfacto_batch_create(dfacto_t* const* jobs, int32_t n, const dfacto
     // Walk configuration: the single-tensor default, then (optionally) tuned.
     C.cfg = choose_walk(C.R, C.dtype, C.nnz, C.m[0].nfib, 0, 0);
     C.cfg.kernel = 2;
-    C.shape = multi_shape_id(C.cfg.vec, C.cfg.G);
     int min_seg = C.cfg.seg;
     int64_t min_P = (int64_t)C.segs() * C.cfg.seg;
     for (const WalkCfg& c : candidates(C)) {

@@ -306,26 +306,29 @@ __global__ void __launch_bounds__(kSortThreads, 3) radix_scatter(
 }
 
 // After the sort: fiber-start flags, duplicate detection, nz_idx and nz_val,
-// and the fiber-end bitmask (bit p of end_bits set iff nonzero p is the last
-// of its fiber: p is the last nonzero or p + 1 starts a new fiber; one ballot
-// per warp of 32 consecutive positions).
+// and the walk's bitmasks (bit p of end_bits set iff nonzero p is the last of
+// its fiber: p is the last nonzero or p + 1 starts a new fiber; bit p of
+// row_bits iff p is the first of its row; one ballot each per warp of 32
+// consecutive positions).
 // narrow: key = (o,f,in) packed with `in` in the low bi bits.
 // wide:   key = (o,f) packed; `in` comes from the COO through perm.
 // With val_payload the payload holds the value's bits (narrow keys), else the
 // nonzero's position in the COO.
 __global__ void segment_flags(const uint64_t* __restrict__ key, const uint32_t* __restrict__ perm,
-                              int64_t n, int bi, bool wide, bool val_payload,
+                              int64_t n, int bf, int bi, bool wide, bool val_payload,
                               const int32_t* __restrict__ idx, int ai,
                               const float* __restrict__ val, int32_t* __restrict__ head,
                               int32_t* __restrict__ nz_idx, float* __restrict__ nz_val,
-                              uint32_t* __restrict__ end_bits, int32_t* __restrict__ dup_flag) {
+                              uint32_t* __restrict__ end_bits, uint32_t* __restrict__ row_bits,
+                              int32_t* __restrict__ dup_flag) {
+  const int so = wide ? bf : bf + bi;  // the key's o starts here
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;  // a multiple of 32
   const int lane = threadIdx.x & 31;
   bool dup = false;
   // warp-uniform loop: the warp's lanes take 32 consecutive positions from p0
   for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); p0 < n; p0 += stride) {
     const int64_t p = p0 + lane;
-    bool endb = false;
+    bool endb = false, rowb = false;
     if (p < n) {
       const uint64_t k = key[p];
       const uint32_t pl = perm[p];
@@ -339,8 +342,10 @@ __global__ void segment_flags(const uint64_t* __restrict__ key, const uint32_t* 
         fkey = shr64(k, bi);
       }
       int32_t h = 1;
+      rowb = true;
       if (p > 0) {
         const uint64_t kp = key[p - 1];
+        rowb = shr64(kp, so) != shr64(k, so);
         if (wide) {
           if (kp == k) {
             h = 0;
@@ -363,7 +368,11 @@ __global__ void segment_flags(const uint64_t* __restrict__ key, const uint32_t* 
       nz_val[p] = val_payload ? __uint_as_float(pl) : val[pl];
     }
     const unsigned bits = __ballot_sync(kFull, endb);
-    if (lane == 0) end_bits[p0 >> 5] = bits;
+    const unsigned rows = __ballot_sync(kFull, rowb);
+    if (lane == 0) {
+      end_bits[p0 >> 5] = bits;
+      row_bits[p0 >> 5] = rows;
+    }
   }
   if (__any_sync(kFull, dup) && lane == 0) atomicOr(dup_flag, 1);
 }
@@ -384,7 +393,10 @@ __global__ void scatter_fibers(const uint64_t* __restrict__ key, const uint32_t*
     fiber_idx[q] = (int32_t)(of & fmask);
     fiber_row[q] = (int32_t)((bf >= 64) ? 0 : (of >> bf));
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) nz_ptr[nfib] = n;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    nz_ptr[nfib] = n;
+    fiber_idx[nfib] = 0;  // past the last fiber: read ahead by the walk, never used
+  }
 }
 
 // fiber_ptr[r] = number of fibers whose row is < r (lower bound in fiber_row).
@@ -401,15 +413,18 @@ __global__ void row_pointers(const int32_t* __restrict__ fiber_row, int64_t nfib
   }
 }
 
-// end_bits: bit e set for the last nonzero e of every fiber, from nz_ptr (the
-// batched tensors' concatenated copies; a tensor's own build sets the bits in
-// segment_flags).
-__global__ void fiber_end_bits(const int64_t* __restrict__ nz_ptr, int64_t nfib,
-                               uint32_t* __restrict__ bits) {
+// Walk bits from the fibers (the batched tensors' concatenated copies; a
+// tensor's own build sets them in segment_flags): bit e of end_bits for the
+// last nonzero e of every fiber, bit p of row_bits for the first nonzero p of
+// every row.
+__global__ void walk_bits(const int64_t* __restrict__ nz_ptr, const int32_t* __restrict__ fiber_row,
+                          int64_t nfib, uint32_t* __restrict__ end_bits,
+                          uint32_t* __restrict__ row_bits) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nfib; q += stride) {
-    const int64_t e = nz_ptr[q + 1] - 1;
-    atomicOr(bits + (e >> 5), 1u << (e & 31));
+    const int64_t p = nz_ptr[q], e = nz_ptr[q + 1] - 1;
+    atomicOr(end_bits + (e >> 5), 1u << (e & 31));
+    if (q == 0 || fiber_row[q - 1] != fiber_row[q]) atomicOr(row_bits + (p >> 5), 1u << (p & 31));
   }
 }
 
@@ -536,13 +551,14 @@ cudaError_t launch_segment_starts(const int64_t* nz_ptr, int64_t nfib, int64_t n
   return cudaGetLastError();
 }
 
-cudaError_t launch_fiber_end_bits(const int64_t* nz_ptr, int64_t nfib, int64_t nnz, uint32_t* bits,
-                                  cudaStream_t s) {
+cudaError_t launch_walk_bits(const int64_t* nz_ptr, const int32_t* fiber_row, int64_t nfib, int64_t nnz,
+                             uint32_t* end_bits, uint32_t* row_bits, cudaStream_t s) {
   const size_t words = (size_t)((nnz + 31) / 32);
   if (words == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(bits, 0, sizeof(uint32_t) * words, s);
+  cudaError_t e = cudaMemsetAsync(end_bits, 0, sizeof(uint32_t) * words, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(row_bits, 0, sizeof(uint32_t) * words, s);
   if (e != cudaSuccess || nfib <= 0) return e;
-  fiber_end_bits<<<grid_for(nfib), 256, 0, s>>>(nz_ptr, nfib, bits);
+  walk_bits<<<grid_for(nfib), 256, 0, s>>>(nz_ptr, fiber_row, nfib, end_bits, row_bits);
   DF_COUNT();
   return cudaGetLastError();
 }
@@ -658,8 +674,18 @@ dfacto_status build_modes(dfacto_t* h, const int32_t* d_idx, const float* d_val)
     const bool wide = !narrow;
     dfacto_status st = DFACTO_OK;
     st = dalloc(h, reinterpret_cast<void**>(&M.fiber_ptr), sizeof(int64_t) * (size_t)(M.dim_o + 1));
-    if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.nz_idx), sizeof(int32_t) * nn);
-    if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.nz_val), sizeof(float) * nn);
+    // zeros up to a multiple of 32 nonzeros (read, and dropped, by the walk)
+    const size_t npad = (size_t)walk_padded(n);
+    if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.nz_idx), sizeof(int32_t) * npad);
+    if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.nz_val), sizeof(float) * npad);
+    if (st == DFACTO_OK && npad > (size_t)n) {
+      e = cudaMemsetAsync(M.nz_idx + n, 0, sizeof(int32_t) * (npad - (size_t)n), s);
+      if (e == cudaSuccess) e = cudaMemsetAsync(M.nz_val + n, 0, sizeof(float) * (npad - (size_t)n), s);
+      if (e != cudaSuccess) {
+        cleanup();
+        return cuda_fail(h, e, "nonzero padding");
+      }
+    }
     if (st != DFACTO_OK) {
       cleanup();
       return st;
@@ -670,6 +696,7 @@ dfacto_status build_modes(dfacto_t* h, const int32_t* d_idx, const float* d_val)
       if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.fiber_idx), sizeof(int32_t));
       if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.fiber_row), sizeof(int32_t));
       if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.end_bits), sizeof(uint32_t));
+      if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.row_bits), sizeof(uint32_t));
       if (st != DFACTO_OK) return st;
       DF_CUDA(h, cudaMemsetAsync(M.nz_ptr, 0, sizeof(int64_t), s));
       DF_CUDA(h, cudaMemsetAsync(M.fiber_ptr, 0, sizeof(int64_t) * (size_t)(M.dim_o + 1), s));
@@ -735,13 +762,14 @@ dfacto_status build_modes(dfacto_t* h, const int32_t* d_idx, const float* d_val)
     prev_bo = bo;
     prev_bf = bf;
     prev_bi = bi;
-    st = dalloc(h, reinterpret_cast<void**>(&M.end_bits), sizeof(uint32_t) * (size_t)((n + 31) / 32));
+    st = dalloc(h, reinterpret_cast<void**>(&M.end_bits), sizeof(uint32_t) * (npad / 32));
+    if (st == DFACTO_OK) st = dalloc(h, reinterpret_cast<void**>(&M.row_bits), sizeof(uint32_t) * (npad / 32));
     if (st != DFACTO_OK) {
       cleanup();
       return st;
     }
-    segment_flags<<<grid_for(n), 256, 0, s>>>(key, perm, n, bi, wide, narrow, d_idx, M.in, d_val,
-                                             head, M.nz_idx, M.nz_val, M.end_bits,
+    segment_flags<<<grid_for(n), 256, 0, s>>>(key, perm, n, bf, bi, wide, narrow, d_idx, M.in, d_val,
+                                             head, M.nz_idx, M.nz_val, M.end_bits, M.row_bits,
                                              h->flags + kFlagDup); DF_COUNT();
     e = cudaGetLastError();
     if (e == cudaSuccess) e = exclusive_scan_i32(head, fid, n, s);
@@ -756,7 +784,7 @@ dfacto_status build_modes(dfacto_t* h, const int32_t* d_idx, const float* d_val)
     M.nfib = (int64_t)last[0] + last[1];
     st = dalloc(h, reinterpret_cast<void**>(&M.nz_ptr), sizeof(int64_t) * (size_t)(M.nfib + 1));
     if (st == DFACTO_OK)
-      st = dalloc(h, reinterpret_cast<void**>(&M.fiber_idx), sizeof(int32_t) * (size_t)M.nfib);
+      st = dalloc(h, reinterpret_cast<void**>(&M.fiber_idx), sizeof(int32_t) * (size_t)(M.nfib + 1));
     if (st == DFACTO_OK)
       st = dalloc(h, reinterpret_cast<void**>(&M.fiber_row), sizeof(int32_t) * (size_t)M.nfib);
     if (st != DFACTO_OK) {

@@ -171,6 +171,46 @@ __global__ void __launch_bounds__(kWalkWarps * 32) dual_walk(const DualParams a)
 // time (their C and GC rows gathered together).  At most 8 values of each of
 // the two gathered rows (B and GB) are in flight per lane.
 // ---------------------------------------------------------------------------
+// A thread's VEC parked floats in shared memory.  Slot k of thread tid holds
+// them as VEC/4 float4 chunks, chunk q at ((k * VEC/4 + q) * NT + tid) * 4, so
+// that a warp's accesses to one chunk are consecutive 16-byte words (no bank
+// conflicts); VEC < 4 keeps the VEC floats together at (k * NT + tid) * VEC.
+template <int VEC, int NT>
+__device__ __forceinline__ float* park_slot(float* vb, int k, int tid) {
+  if constexpr (VEC % 4 == 0) return vb + ((size_t)k * (VEC / 4) * NT + tid) * 4;
+  else return vb + ((size_t)k * NT + tid) * VEC;
+}
+template <int VEC, int NT>
+__device__ __forceinline__ void smem_st(float* p, const float (&v)[VEC]) {
+  if constexpr (VEC % 4 == 0) {
+#pragma unroll
+    for (int e = 0; e < VEC; e += 4)
+      *reinterpret_cast<float4*>(p + (size_t)(e / 4) * NT * 4) =
+          make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+  } else if constexpr (VEC == 2) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) p[e] = v[e];
+  }
+}
+template <int VEC, int NT>
+__device__ __forceinline__ void smem_ld(const float* p, float (&v)[VEC]) {
+  if constexpr (VEC % 4 == 0) {
+#pragma unroll
+    for (int e = 0; e < VEC; e += 4) {
+      const float4 t = *reinterpret_cast<const float4*>(p + (size_t)(e / 4) * NT * 4);
+      v[e] = t.x; v[e + 1] = t.y; v[e + 2] = t.z; v[e + 3] = t.w;
+    }
+  } else if constexpr (VEC == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) v[e] = p[e];
+  }
+}
+
 template <int VEC>
 struct Dual2Shape {
   static constexpr int NT = kWalkWarps * 32;
@@ -447,10 +487,6 @@ dfacto_status dual_pass(dfacto_t* h) {
   const int RP = walk_rank(R, h->opt.vec);
   const bool padded = RP != R;
   WalkCfg cfg = M.cfg;
-  if (padded) {
-    cfg = choose_walk(RP, DFACTO_F32, h->nnz, M.nfib, h->opt.seg_nnz, 0);
-    cfg.kernel = M.cfg.kernel;
-  }
   if (cfg.kernel == 2 && cfg.vec > 4) {
     cfg.vec = 4;
     int G = 1;

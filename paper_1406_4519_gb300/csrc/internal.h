@@ -39,12 +39,13 @@ struct ModeCSR {
   int64_t dim_o = 0;
   int64_t nfib = 0;
   int64_t* fiber_ptr = nullptr;  // [dim_o + 1]  row(M^r)
-  int32_t* fiber_idx = nullptr;  // [nfib]       col(M^r) = f
+  int32_t* fiber_idx = nullptr;  // [nfib] (+ 1 unused) col(M^r) = f
   int32_t* fiber_row = nullptr;  // [nfib]       o of each fiber (COO form of row(M^r))
   int64_t* nz_ptr = nullptr;     // [nfib + 1]
-  int32_t* nz_idx = nullptr;     // [nnz]        index `in`
-  float* nz_val = nullptr;       // [nnz]
+  int32_t* nz_idx = nullptr;     // [nnz]        index `in` (zeros up to a multiple of 32)
+  float* nz_val = nullptr;       // [nnz]        (zeros up to a multiple of 32)
   uint32_t* end_bits = nullptr;  // [(nnz + 31) / 32] bit p set iff nonzero p ends its fiber
+  uint32_t* row_bits = nullptr;  // [(nnz + 31) / 32] bit p set iff nonzero p starts its row
   WalkCfg cfg;
   int64_t nseg = 0;              // segments of cfg.seg nonzeros
   int32_t* seg_fib = nullptr;    // [nseg] fiber holding the first nonzero of each segment

@@ -10,6 +10,11 @@ namespace {
 
 constexpr int kFixThreads = 256;
 constexpr int kFixWarps = kFixThreads / 32;
+// Waves of walk CTAs (152 SMs, two resident) below which segments get shorter:
+// two, measured against one and four (5M uniform nonzeros, R = 16, BF16: 96 us
+// per mode against 106 and 105; the same within 1% on 1M to 60M power-law
+// nonzeros).
+constexpr int kWalkWaves = 2;
 constexpr int kAheadCols = 32;  // carry values per lane a warp loads before adding them
 
 // One block per CTA c (grid-stride): if c's last partial run belongs to a row r
@@ -168,7 +173,6 @@ cudaError_t launch_mttkrp_fixup(const int32_t* carry_row, const float* carry,
 }
 
 WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, int vec_opt) {
-  (void)nnz;
   (void)nfib;
   WalkCfg c;
   // Default: one 16-byte load per lane and factor row (4 FP32 or 8 BF16
@@ -184,7 +188,18 @@ WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, in
   c.vec = vec;
   c.G = G;
   c.kernel = 2;  // fiber ends from the end bitmask (faster on every measured shape)
-  int seg = seg_opt > 0 ? seg_opt : 128;
+  
+  // Segment length: a CTA's fixed cost (its first dependent loads and the merge
+  // of its partial rows) is paid per segment, so long segments are better as
+  // long as the CTAs fill the GPU kWalkWaves times over (50M power-law
+  // nonzeros, R = 16: 530 us per mode with segments of 128, 514 with 256; 10,000
+  // uniform nonzeros, R = 10: 39 us with 128, 29 with 32).
+  const int segs = kWalkWarps * (32 / G);
+  int seg = seg_opt;
+  if (seg <= 0) {
+    seg = 256;
+    while (seg > 32 && nnz < (int64_t)segs * seg * kWalkWaves * 152 * 2) seg >>= 1;
+  }
   seg = std::max(32, (seg + 31) / 32 * 32);
   c.seg = seg;
   return c;
@@ -201,11 +216,7 @@ dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out) {
   const int R = h->R;
   const int RP = walk_rank(R, h->opt.vec);
   const bool padded = RP != R;
-  WalkCfg cfg = M.cfg;
-  if (padded) {
-    cfg = choose_walk(RP, DFACTO_F32, h->nnz, M.nfib, h->opt.seg_nnz, 0);
-    cfg.kernel = M.cfg.kernel;
-  }
+  const WalkCfg cfg = M.cfg;
   dfacto_status st = ensure_segments(h, mode);
   if (st != DFACTO_OK) return st;
   const int segs = kWalkWarps * (32 / cfg.G);
@@ -250,6 +261,7 @@ dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out) {
   a.nz_val = M.nz_val;
   a.seg_fib = M.seg_fib;
   a.end_bits = M.end_bits;
+  a.row_bits = M.row_bits;
   a.Fin = Fin;
   a.Ff = Ff;
   a.out = wout;

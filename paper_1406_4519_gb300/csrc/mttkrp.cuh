@@ -23,6 +23,8 @@
 // therefore has a fixed order: results are bitwise reproducible.
 #pragma once
 
+#include <type_traits>
+
 #include "device.cuh"
 #include "internal.h"
 
@@ -37,6 +39,7 @@ struct MttkrpParams {
   const float* nz_val;
   const int32_t* seg_fib;
   const uint32_t* end_bits;  // bit p set iff nonzero p ends its fiber (walk2)
+  const uint32_t* row_bits;  // bit p set iff nonzero p starts its row (walk2)
   const void* Fin;
   const void* Ff;
   float* out;
@@ -378,86 +381,183 @@ __global__ void __launch_bounds__(kWalkWarps * 32) mttkrp_walk(const MttkrpParam
 }
 
 // ---------------------------------------------------------------------------
-// mttkrp_walk2: the same walk with fiber ends taken from a bitmask and fibers
-// closed in batches.  Per sub-batch of U steps a group
-//   (1) gathers the U F_in rows,
-//   (2) accumulates v over the U nonzeros; where a bit of end_bits marks the
-//       last nonzero of a fiber, v is parked in a per-lane shared-memory slot
-//       and restarted (no branch on fiber metadata in this loop),
-//   (3) closes the k <= U fibers that ended: loads their f and row, issues all
-//       k F_f gathers at once, then folds v_j (*) F_f[f_j] into the row sums.
-// The merge of rows shared between segments, warps and CTAs is the one of
-// mttkrp_walk.
+// mttkrp_walk2: the same sums in the same order with no branch on fiber
+// metadata.  end_bits and row_bits mark the nonzeros that end a fiber and that
+// start a row.  A group takes its segment in batches of B positions, whose
+// (in, x) its lanes hold LPP each (loaded one batch ahead); the fiber of a
+// position is the batch's first fiber plus the number of end bits before it,
+// so each lane also holds f of its positions' fibers.  Per sub-batch of U
+// positions the group gathers the U F_in rows and the F_f rows of the fibers
+// that end there together, all independent of one another, and runs
+//   v += x F_in;  at a fiber's last nonzero: acc += v (*) F_f, v = 0
+// as predicated arithmetic; (in, x, f) are passed around by shuffles.  Batches
+// in which no group of the warp starts a row (most of them on power-law
+// tensors) skip the row tests.  The merge of rows shared between segments,
+// warps and CTAs is the one of mttkrp_walk.
+//
+// What bounds it: the latency of the gathers against the registers that hold
+// them.  The gathers mostly hit L1 and L2 (a bare probe of 128-byte rows reaches
+// 140 G rows/s from L2 on this GPU, the walk 80 on 50M power-law nonzeros at
+// R = 32), so what counts is how many are in flight and how few instructions
+// stand between two rounds: the earlier form of this walk parked the fiber sums
+// in shared memory and folded them in a second, dependent round of loads (18
+// warp instructions per nonzero, now 9).  Per mode of 50M power-law nonzeros,
+// before and now: R = 32 1.05 and 0.85 ms, R = 16 0.64 and 0.52, R = 8 0.59 and
+// 0.40, R = 32 with BF16 factors 1.04 and 0.56.  Slower here: the streams
+// staged in shared memory by cp.async (0.87 ms at R = 32, 12 instructions), the
+// sum taken term by term without fibers (0.80 ms at R = 32 but 1.1 times slower
+// at R = 12 to 16, and a gather more per nonzero), and eight FP32 columns per
+// lane.
+//
+// nz_idx, nz_val and the bit words are allocated up to a multiple of 32
+// nonzeros, zero past nnz: those positions read row 0, and as they end no
+// fiber what they add to v is dropped.  fiber_idx has one entry more than
+// fibers (the fiber "after" the last one, never gathered).  Lanes past column
+// R walk column 0 and store nothing.
 // ---------------------------------------------------------------------------
-// A thread's VEC parked floats in shared memory.  Slot k of thread tid holds
-// them as VEC/4 float4 chunks, chunk q at ((k * VEC/4 + q) * NT + tid) * 4, so
-// that a warp's accesses to one chunk are consecutive 16-byte words (no bank
-// conflicts); VEC < 4 keeps the VEC floats together at (k * NT + tid) * VEC.
-template <int VEC, int NT>
-__device__ __forceinline__ float* park_slot(float* vb, int k, int tid) {
-  if constexpr (VEC % 4 == 0) return vb + ((size_t)k * (VEC / 4) * NT + tid) * 4;
-  else return vb + ((size_t)k * NT + tid) * VEC;
-}
-template <int VEC, int NT>
-__device__ __forceinline__ void smem_st(float* p, const float (&v)[VEC]) {
-  if constexpr (VEC % 4 == 0) {
+
+// VEC FP32 columns of a lane, two to a 64-bit register (one FFMA2 per pair).
+template <int VEC>
+struct Cols {
+  uint64_t p[VEC / 2];
+  __device__ __forceinline__ void zero() {
 #pragma unroll
-    for (int e = 0; e < VEC; e += 4)
-      *reinterpret_cast<float4*>(p + (size_t)(e / 4) * NT * 4) =
-          make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-  } else if constexpr (VEC == 2) {
-    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    for (int e = 0; e < VEC / 2; ++e) p[e] = 0ull;
+  }
+  __device__ __forceinline__ void unpack(float (&o)[VEC]) const {
+#pragma unroll
+    for (int e = 0; e < VEC / 2; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(o[2 * e]), "=f"(o[2 * e + 1]) : "l"(p[e]));
+  }
+};
+template <>
+struct Cols<1> {
+  float p[1];
+  __device__ __forceinline__ void zero() { p[0] = 0.f; }
+  __device__ __forceinline__ void unpack(float (&o)[1]) const { o[0] = p[0]; }
+};
+
+// v += x w.
+template <int VEC>
+__device__ __forceinline__ void axpy_cols(float x, const Cols<VEC>& w, Cols<VEC>& v) {
+  if constexpr (VEC == 1) {
+    v.p[0] = fmaf(x, w.p[0], v.p[0]);
   } else {
+    uint64_t xx;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x));
 #pragma unroll
-    for (int e = 0; e < VEC; ++e) p[e] = v[e];
+    for (int e = 0; e < VEC / 2; ++e) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v.p[e]) : "l"(xx), "l"(w.p[e]));
   }
 }
-template <int VEC, int NT>
-__device__ __forceinline__ void smem_ld(const float* p, float (&v)[VEC]) {
-  if constexpr (VEC % 4 == 0) {
+
+// If `on` is nonzero: acc += v w, v = 0 (predicated, no branch).
+template <int VEC>
+__device__ __forceinline__ void fold_cols_if(uint32_t on, const Cols<VEC>& w, Cols<VEC>& v, Cols<VEC>& acc) {
+  if constexpr (VEC == 1) {
+    asm("{.reg .pred q;\nsetp.ne.u32 q, %3, 0;\n@q fma.rn.f32 %0, %1, %2, %0;\n@q mov.f32 %1, 0f00000000;}"
+        : "+f"(acc.p[0]), "+f"(v.p[0])
+        : "f"(w.p[0]), "r"(on));
+  } else {
 #pragma unroll
-    for (int e = 0; e < VEC; e += 4) {
-      const float4 t = *reinterpret_cast<const float4*>(p + (size_t)(e / 4) * NT * 4);
-      v[e] = t.x; v[e + 1] = t.y; v[e + 2] = t.z; v[e + 3] = t.w;
+    for (int e = 0; e < VEC / 2; ++e)
+      asm("{.reg .pred q;\n.reg .f32 a0, a1, v0, v1, w0, w1;\nsetp.ne.u32 q, %3, 0;\n"
+          "mov.b64 {a0, a1}, %0;\nmov.b64 {v0, v1}, %1;\nmov.b64 {w0, w1}, %2;\n"
+          "@q fma.rn.f32 a0, v0, w0, a0;\n@q fma.rn.f32 a1, v1, w1, a1;\n"
+          "@q mov.f32 v0, 0f00000000;\n@q mov.f32 v1, 0f00000000;\n"
+          "mov.b64 %0, {a0, a1};\nmov.b64 %1, {v0, v1};}"
+          : "+l"(acc.p[e]), "+l"(v.p[e])
+          : "l"(w.p[e]), "r"(on));
+  }
+}
+
+// VEC consecutive entries of a factor row as they are stored (widened at use).
+template <typename T, int VEC>
+struct RawCols;
+template <int VEC>
+struct RawCols<float, VEC> {
+  Cols<VEC> v;
+  __device__ __forceinline__ void load(const float* p) {
+    if constexpr (VEC == 8) {
+      asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v.p[0]), "=l"(v.p[1]), "=l"(v.p[2]), "=l"(v.p[3]) : "l"(p));
+    } else if constexpr (VEC == 4) {
+      asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(v.p[0]), "=l"(v.p[1]) : "l"(p));
+    } else if constexpr (VEC == 2) {
+      asm("ld.global.nc.b64 %0, [%1];" : "=l"(v.p[0]) : "l"(p));
+    } else {
+      v.p[0] = __ldg(p);
     }
-  } else if constexpr (VEC == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(p);
-    v[0] = t.x; v[1] = t.y;
-  } else {
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) v[e] = p[e];
   }
-}
+  __device__ __forceinline__ Cols<VEC> get() const { return v; }
+};
+template <int VEC>
+struct RawCols<__nv_bfloat16, VEC> {
+  uint32_t w[(VEC + 1) / 2];
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) {
+    if constexpr (VEC == 8) {
+      const uint4 t = __ldg(reinterpret_cast<const uint4*>(p));
+      w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+    } else if constexpr (VEC == 4) {
+      const uint2 t = __ldg(reinterpret_cast<const uint2*>(p));
+      w[0] = t.x; w[1] = t.y;
+    } else if constexpr (VEC == 2) {
+      w[0] = __ldg(reinterpret_cast<const unsigned int*>(p));
+    } else {
+      w[0] = __ldg(reinterpret_cast<const unsigned short*>(p));
+    }
+  }
+  __device__ __forceinline__ Cols<VEC> get() const {
+    Cols<VEC> o;
+    if constexpr (VEC == 1) {
+      o.p[0] = bf16_lo(w[0]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < VEC / 2; ++e)
+        asm("mov.b64 %0, {%1, %2};" : "=l"(o.p[e]) : "f"(bf16_lo(w[e])), "f"(bf16_hi(w[e])));
+    }
+    return o;
+  }
+};
 
-// Fibers closed per round of the fiber-closing pass (fewer predicated-off
-// slots when fibers are long; a sub-batch closes at most U).
-constexpr int kCloseChunk = 4;
+// Positions of the nonzero arrays a tensor of nnz nonzeros allocates.
+__host__ __device__ constexpr int64_t walk_padded(int64_t nnz) { return (nnz + 31) / 32 * 32; }
 
-// Gathers in flight per lane of the walk shape (VEC, G): at most 16 gathered
-// values (U * VEC <= 16); more leave the kernel short of registers (spills) at
-// the budget of Walk2Shape.
-__host__ __device__ constexpr int walk2_gathers(int vec, int G) { return G < 16 / vec ? G : 16 / vec; }
-// Per-lane shared-memory slots for parked fiber sums.
-__host__ __device__ constexpr int walk2_park_slots(int vec, int G) { return walk2_gathers(vec, G); }
 // Dynamic shared memory of the walk at rank R: segment and warp partial rows
-// for the merge, then the park slots.
-inline size_t walk2_smem_bytes(int vec, int G, int R) {
-  return sizeof(float) * ((size_t)(2 * kWalkWarps * (32 / G) + 2 * kWalkWarps) * R +
-                          (size_t)kWalkWarps * 32 * walk2_park_slots(vec, G) * vec);
+// for the merge.
+inline size_t walk2_smem_bytes(int G, int R) {
+  return sizeof(float) * (size_t)(2 * kWalkWarps * (32 / G) + 2 * kWalkWarps) * R;
 }
 
 template <typename T, int VEC, int G>
 struct Walk2Shape {
   static constexpr int NG = 32 / G;
   static constexpr int SEGS = kWalkWarps * NG;
-  static constexpr int U = walk2_gathers(VEC, G);
-  // Resident CTAs per SM the register budget is cut for: the kernel is bound by
-  // the latency of its gathers and its L1 traffic, so occupancy pays more than
-  // a few registers: 80 registers (3 CTAs) for eight-column lanes, 64 (4 CTAs)
-  // for narrower ones.
-  static constexpr int MIN_BLOCKS = VEC >= 8 ? 3 : 4;
-  static size_t smem_bytes(int R) { return walk2_smem_bytes(VEC, G, R); }
+  // Positions per lane and batch, and per batch (divides 32).
+  static constexpr int LPP = G >= 8 ? 1 : (G == 4 || VEC >= 8 ? 2 : 4);
+  static constexpr int B = G * LPP;
+  // Two buffers of U gathered rows and a budget of 128 registers (two CTAs per
+  // SM): while one buffer is used the other is filled.  Eight lanes of four FP32
+  // columns (R = 32) do better with one buffer at 80 registers and three CTAs.
+  static constexpr int REGS = (VEC * (int)sizeof(T) + 3) / 4;  // registers of a row
+  static constexpr int NBUF = REGS == 4 && VEC == 4 && G == 8 ? 1 : 2;
+  static constexpr int MIN_BLOCKS = NBUF == 1 ? 3 : 2;
+  static constexpr int U0 = REGS >= 8 ? 2 : (REGS >= 4 ? 4 : 8);
+  static constexpr int U = NBUF * U0 <= B ? U0 : (B >= NBUF ? B / NBUF : 1);
+  static_assert(B % (NBUF * U) == 0 && 32 % B == 0, "batch layout");
+  static size_t smem_bytes(int R) { return walk2_smem_bytes(G, R); }
 };
+
+// LPP consecutive 32-bit words (the address is a multiple of their size).
+template <int LPP>
+__device__ __forceinline__ void ldg_words(const int32_t* p, int (&o)[LPP]) {
+  if constexpr (LPP == 4) {
+    const int4 t = __ldg(reinterpret_cast<const int4*>(p));
+    o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+  } else if constexpr (LPP == 2) {
+    const int2 t = __ldg(reinterpret_cast<const int2*>(p));
+    o[0] = t.x; o[1] = t.y;
+  } else {
+    o[0] = __ldg(p);
+  }
+}
 
 // The walk of CTA `cta` of one MTTKRP (shared by the single-tensor kernel and
 // the batched one).  smem holds Walk2Shape::smem_bytes(R) bytes; s_row and
@@ -466,12 +566,11 @@ template <typename T, int VEC, int G>
 __device__ __forceinline__ void walk2_cta(const MttkrpParams& a, int cta, float* smem,
                                           int32_t* s_row, int32_t* w_row) {
   using Shape = Walk2Shape<T, VEC, G>;
-  constexpr int NG = Shape::NG, SEGS = Shape::SEGS, U = Shape::U;
-  constexpr int NT = kWalkWarps * 32;
+  constexpr int NG = Shape::NG, SEGS = Shape::SEGS, U = Shape::U, LPP = Shape::LPP, B = Shape::B;
+  constexpr uint32_t kBatch = B == 32 ? 0xffffffffu : (1u << (B & 31)) - 1u;
   const int R = a.R;
-  float* s_val = smem;                           // [SEGS * 2][R]
-  float* w_val = smem + (size_t)SEGS * 2 * R;    // [kWalkWarps * 2][R]
-  float* vb = w_val + (size_t)kWalkWarps * 2 * R;  // U slots of NT x VEC parked fiber sums
+  float* s_val = smem;                         // [SEGS * 2][R]
+  float* w_val = smem + (size_t)SEGS * 2 * R;  // [kWalkWarps * 2][R]
 
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
@@ -480,147 +579,152 @@ __device__ __forceinline__ void walk2_cta(const MttkrpParams& a, int cta, float*
   const int col0 = c * VEC;
   const bool colok = col0 < R;
   const int sl = warp * NG + g;
-  // Positions fit in int: nnz <= kMaxNnz and seg <= kMaxSeg keep p0 + seg + G
+  // Positions fit in int: nnz <= kMaxNnz and seg <= kMaxSeg keep p0 + seg + 32
   // below 2^31 (the bounds are formed in 64 bits first).
   const int nnz = (int)a.nnz;
+  const int npad = (int)walk_padded(a.nnz);
   const int cta_p0 = (int)min((int64_t)cta * SEGS * a.seg, a.nnz);
   const int cta_p1 = (int)min((int64_t)cta_p0 + (int64_t)SEGS * a.seg, a.nnz);
-  const int p0 = (int)min((int64_t)cta_p0 + (int64_t)sl * a.seg, a.nnz);
+  const int p0 = (int)min((int64_t)cta * SEGS * a.seg + (int64_t)sl * a.seg, (int64_t)npad);
   const int p1 = min(p0 + a.seg, nnz);
   const bool active = p0 < nnz;
-  const T* __restrict__ Fin = static_cast<const T*>(a.Fin);
-  const T* __restrict__ Ff = static_cast<const T*>(a.Ff);
+  // row t of the gathered factors from the lane's first column on
+  const char* Fin = reinterpret_cast<const char*>(static_cast<const T*>(a.Fin) + (colok ? col0 : 0));
+  const char* Ff = reinterpret_cast<const char*>(static_cast<const T*>(a.Ff) + (colok ? col0 : 0));
+  const uint32_t stride = (uint32_t)(R * (int)sizeof(T));
+  auto row_of = [&](const char* F, int t) {
+    return reinterpret_cast<const T*>(F + (uint64_t)(uint32_t)t * stride);
+  };
 
-  float v[VEC], acc[VEC];
-#pragma unroll
-  for (int k = 0; k < VEC; ++k) { v[k] = 0.f; acc[k] = 0.f; }
-  int q = 0;          // fiber holding the current nonzero
+  Cols<VEC> v, acc;
+  v.zero();
+  acc.zero();
+  int q = 0;  // fiber holding the batch's first position
   int row_cur = -1;
+  uint32_t ew = 0u, rw = 0u;  // end and row-start bits from the batch's first position on
   if (active) {
     q = a.seg_fib[(int64_t)cta * SEGS + sl];
     row_cur = a.fiber_row[q];
+    ew = __ldg(a.end_bits + (p0 >> 5));
+    rw = __ldg(a.row_bits + (p0 >> 5)) & ~1u;  // the segment's first row is row_cur
   }
-  bool head_open = true;
-  auto put_slot = [&](int k, int row, const float (&val)[VEC]) {
-    if (c == 0) s_row[sl * 2 + k] = row;
+  // Segment slots: 0 = head row partial, 1 = tail row partial (-1 = none).  A
+  // finished row goes to the output, the segment's first row to slot 0 (a
+  // generic address either way).
+  if (c == 0) s_row[sl * 2] = row_cur;
+  float* head = s_val + (size_t)(sl * 2) * R + col0;  // null once the first row is in its slot
+  auto put_row = [&](float* dst) {
     if (colok) {
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) s_val[(size_t)(sl * 2 + k) * R + col0 + e] = val[e];
+      float val[VEC];
+      acc.unpack(val);
+      VecIO<float, VEC>::store(dst, val);
     }
   };
-  // Fold w = vv (*) ff of a fiber of row r into the row sums (emitting the
-  // previous row when r starts a new one).
-  auto fold = [&](int r, const float (&vv)[VEC], const float (&ff)[VEC]) {
-    if (r != row_cur) {
-      if (head_open) {
-        put_slot(0, row_cur, acc);
-        head_open = false;
-      } else if (colok) {
-        VecIO<float, VEC>::store(a.out + (int64_t)row_cur * R + col0, acc);
-      }
+  // The lane's positions of the batch at p (past the arrays: of their last
+  // batch, whose values are then not used).
+  auto load_stream = [&](int p, int (&in)[LPP], int (&x)[LPP]) {
+    const int pl = min(p, npad - B) + c * LPP;
+    ldg_words<LPP>(a.nz_idx + pl, in);
+    ldg_words<LPP>(reinterpret_cast<const int32_t*>(a.nz_val) + pl, x);
+  };
+  // f of the fibers of the lane's positions of a batch that starts in fiber qb.
+  auto load_fibers = [&](int qb, uint32_t e, int (&f)[LPP]) {
 #pragma unroll
-      for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
-      row_cur = r;
-    }
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) acc[e] = fmaf(vv[e], ff[e], acc[e]);
+    for (int j = 0; j < LPP; ++j)
+      f[j] = __ldg(a.fiber_idx + (qb + __popc(e & ((1u << (c * LPP + j)) - 1u))));
   };
 
-  for (int base = p0; base < p0 + a.seg; base += G) {
-    const int pl = base + c;
-    const bool okl = pl < p1;
-    const int my_in = okl ? __ldg(a.nz_idx + pl) : 0;
-    const float my_x = okl ? __ldg(a.nz_val + pl) : 0.f;
-    // end bits of the batch's G positions (base is a multiple of G, G | 32);
-    // a batch starting at or past p1 has none, and its word may lie past the
-    // end of end_bits ((nnz + 31) / 32 words) in the last segment
-    const uint32_t ebits = (active && base < p1) ? (__ldg(a.end_bits + (base >> 5)) >> (base & 31)) : 0u;
+  // Gather the rows of positions u0 .. u0 + U - 1 of a batch (in, f, end bits).
+  struct Rows {
+    RawCols<T, VEC> fin[U], ff[U];
+  };
+  auto issue = [&](Rows& w, int u0, const int (&in)[LPP], const int (&f)[LPP], uint32_t e) {
 #pragma unroll
-    for (int u0 = 0; u0 < G; u0 += U) {
-      float fin[U][VEC];
+    for (int uu = 0; uu < U; ++uu) {
+      const int iu = G == 1 ? in[(u0 + uu) % LPP] : __shfl_sync(kFull, in[(u0 + uu) % LPP], gbase + (u0 + uu) / LPP);
+      w.fin[uu].load(row_of(Fin, iu));
+    }
 #pragma unroll
-      for (int uu = 0; uu < U; ++uu) {
-        const int in = __shfl_sync(kFull, my_in, gbase + u0 + uu);
-        if (colok && base + u0 + uu < p1) {
-          VecIO<T, VEC>::load(Fin + (int64_t)in * R + col0, fin[uu]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) fin[uu][e] = 0.f;
-        }
+    for (int uu = 0; uu < U; ++uu) {
+      const int fu = G == 1 ? f[(u0 + uu) % LPP] : __shfl_sync(kFull, f[(u0 + uu) % LPP], gbase + (u0 + uu) / LPP);
+      if (e & (1u << (u0 + uu))) w.ff[uu].load(row_of(Ff, fu));
+    }
+  };
+
+  int in[LPP], x[LPP], f[LPP];
+  load_stream(p0, in, x);
+  load_fibers(q, ew, f);
+  Rows buf[Shape::NBUF];
+  if constexpr (Shape::NBUF == 2) issue(buf[0], 0, in, f, ew);
+  for (int pb = p0; pb < p0 + a.seg; pb += 32) {
+    uint32_t ewn = 0u, rwn = 0u;  // the next 32 positions' bits
+    if (pb + 32 < p1) {
+      ewn = __ldg(a.end_bits + ((pb + 32) >> 5));
+      rwn = __ldg(a.row_bits + ((pb + 32) >> 5));
+    }
+#pragma unroll 1
+    for (int k = 0; k < 32 / B; ++k) {
+      const uint32_t eb = ew & kBatch, rb = rw & kBatch;
+      const int qn = q + __popc(eb);
+      if constexpr (B < 32) {
+        ew = k == 32 / B - 1 ? ewn : ew >> (B & 31);
+        rw = k == 32 / B - 1 ? rwn : rw >> (B & 31);
+      } else {
+        ew = ewn;
+        rw = rwn;
       }
-      int k = 0;  // fibers closed in this sub-batch
+      int in_n[LPP], x_n[LPP], f_n[LPP];
+      load_stream(pb + (k + 1) * B, in_n, x_n);
+      load_fibers(qn, ew, f_n);
+      const bool any = __any_sync(kFull, rb != 0u);
+      auto batch = [&](auto with_rows) {
 #pragma unroll
-      for (int uu = 0; uu < U; ++uu) {
-        const float x = __shfl_sync(kFull, my_x, gbase + u0 + uu);
-        const int p = base + u0 + uu;
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) v[e] = fmaf(x, fin[uu][e], v[e]);
-        const bool end = p < p1 && ((ebits >> (u0 + uu)) & 1u);
-        if (end) {
-          smem_st<VEC, NT>(park_slot<VEC, NT>(vb, k, tid), v);
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) v[e] = 0.f;
-        }
-        k += end ? 1 : 0;
-      }
-      // Close the k fibers q .. q + k - 1, CC at a time (the F_f gathers of a
-      // round are issued together).
-      constexpr int CC = kCloseChunk < U ? kCloseChunk : U;
-      for (int j0 = 0; j0 < k; j0 += CC) {
-        int fj[CC], rj[CC];
-#pragma unroll
-        for (int j = 0; j < CC; ++j) {
-          fj[j] = 0;
-          rj[j] = row_cur;
-          if (j0 + j < k) {
-            fj[j] = __ldg(a.fiber_idx + q + j0 + j);
-            rj[j] = __ldg(a.fiber_row + q + j0 + j);
-          }
-        }
-        float ff[CC][VEC];
-#pragma unroll
-        for (int j = 0; j < CC; ++j) {
-          if (j0 + j < k && colok) {
-            VecIO<T, VEC>::load(Ff + (int64_t)fj[j] * R + col0, ff[j]);
+        for (int u0 = 0; u0 < B; u0 += U) {
+          if constexpr (Shape::NBUF == 2) {
+            // the next positions' rows are on their way while these are used
+            if (u0 + U < B) issue(buf[((u0 / U) + 1) % 2], u0 + U, in, f, eb);
+            else issue(buf[((u0 / U) + 1) % 2], 0, in_n, f_n, ew);
           } else {
+            issue(buf[0], u0, in, f, eb);
+          }
+          const Rows& now = buf[(u0 / U) % Shape::NBUF];
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) ff[j][e] = 0.f;
+          for (int uu = 0; uu < U; ++uu) {
+            const int u = u0 + uu;
+            const float xu = __int_as_float(G == 1 ? x[u % LPP] : __shfl_sync(kFull, x[u % LPP], gbase + u / LPP));
+            if constexpr (decltype(with_rows)::value) {
+              if ((rb >> u) & 1u) {
+                put_row(head ? head : a.out + (int64_t)row_cur * R + col0);
+                head = nullptr;
+                acc.zero();
+                row_cur = __ldg(a.fiber_row + (q + __popc(eb & ((1u << u) - 1u))));
+              }
+            }
+            axpy_cols<VEC>(xu, now.fin[uu].get(), v);
+            fold_cols_if<VEC>(eb & (1u << u), now.ff[uu].get(), v, acc);
           }
         }
+      };
+      if (any) batch(std::true_type{});
+      else batch(std::false_type{});
+      q = qn;
 #pragma unroll
-        for (int j = 0; j < CC; ++j) {
-          if (j0 + j < k) {
-            float vv[VEC];
-            smem_ld<VEC, NT>(park_slot<VEC, NT>(vb, j0 + j, tid), vv);
-            fold(rj[j], vv, ff[j]);
-          }
-        }
+      for (int j = 0; j < LPP; ++j) {
+        in[j] = in_n[j];
+        x[j] = x_n[j];
+        f[j] = f_n[j];
       }
-      q += k;
     }
   }
   // The fiber open at the segment end (if its last nonzero lies beyond p1).
   if (active && !((__ldg(a.end_bits + ((p1 - 1) >> 5)) >> ((p1 - 1) & 31)) & 1u)) {
-    const int f = __ldg(a.fiber_idx + q);
-    const int r = __ldg(a.fiber_row + q);
-    float ff[VEC];
-    if (colok) VecIO<T, VEC>::load(Ff + (int64_t)f * R + col0, ff);
-    else {
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) ff[e] = 0.f;
-    }
-    fold(r, v, ff);
+    RawCols<T, VEC> ff;
+    ff.load(row_of(Ff, __ldg(a.fiber_idx + q)));
+    fold_cols_if<VEC>(1u, ff.get(), v, acc);
   }
 
-  // Segment slots: 0 = head row partial, 1 = tail row partial (-1 = none).
-  if (!active) {
-    if (c == 0) { s_row[sl * 2] = -1; s_row[sl * 2 + 1] = -1; }
-  } else if (head_open) {
-    put_slot(0, row_cur, acc);
-    if (c == 0) s_row[sl * 2 + 1] = -1;
-  } else {
-    put_slot(1, row_cur, acc);
-  }
+  if (c == 0) s_row[sl * 2 + 1] = head ? -1 : row_cur;
+  if (active) put_row(s_val + (size_t)(sl * 2 + (head ? 0 : 1)) * R + col0);
   __syncthreads();
   mttkrp_merge_cta<SEGS, NG>(a, cta, s_row, s_val, w_row, w_val, lane, warp, cta_p0, cta_p1);
 }
@@ -635,67 +739,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32, (Walk2Shape<T, VEC, G>::MIN_B
   walk2_cta<T, VEC, G>(a, blockIdx.x, smem, s_row, w_row);
 }
 
-// ---------------------------------------------------------------------------
-// Batched MTTKRP: the jobs of a batch that share (R, factor type) form one
-// block-diagonal tensor (a "rank class": indices offset per job, factors
-// pooled), so a class is one walk.  mttkrp_walk2_multi walks up to
-// kMaxClasses classes in one persistent launch: block b takes the virtual CTAs
-// b, b + gridDim.x, ... of the concatenated class ranges, and each class runs
-// the walk shape its autotuned (VEC, G) selects.  The per-class parameters stay
-// in the kernel's parameter space (__grid_constant__).
-// ---------------------------------------------------------------------------
-constexpr int kMaxClasses = 4;
-
-// Walk shapes compiled into the batched kernel: (VEC, G) by id.
-constexpr int kMultiShapes = 6;
-__host__ __device__ constexpr int multi_shape_vec(int id) { return id < 3 ? 4 : 8; }
-__host__ __device__ constexpr int multi_shape_G(int id) {
-  return id == 0 ? 2 : id == 1 ? 4 : id == 2 ? 8 : id == 3 ? 1 : id == 4 ? 2 : 4;
-}
-inline int multi_shape_id(int vec, int G) {
-  for (int i = 0; i < kMultiShapes; ++i)
-    if (multi_shape_vec(i) == vec && multi_shape_G(i) == G) return i;
-  return -1;
-}
-constexpr int kMultiMaxSegs = kWalkWarps * 32;  // SEGS of the G = 1 shape
-
-struct MultiWalkParams {
-  MttkrpParams p[kMaxClasses];
-  int shape[kMaxClasses];          // multi shape id of each class
-  int cta_begin[kMaxClasses + 1];  // virtual CTAs [cta_begin[c], cta_begin[c + 1]) walk class c
-  int nclass;
-};
-
-template <typename T>
-__global__ void __launch_bounds__(kWalkWarps * 32, 3)
-    mttkrp_walk2_multi(const __grid_constant__ MultiWalkParams mp) {
-  extern __shared__ __align__(16) float smem[];
-  __shared__ int32_t s_row[kMultiMaxSegs * 2];
-  __shared__ int32_t w_row[kWalkWarps * 2];
-  const int total = mp.cta_begin[mp.nclass];
-  for (int v = blockIdx.x; v < total; v += gridDim.x) {
-    int c = 0;
-#pragma unroll
-    for (int k = 1; k < kMaxClasses; ++k)
-      if (k < mp.nclass && v >= mp.cta_begin[k]) c = k;
-    const MttkrpParams& a = mp.p[c];
-    const int cta = v - mp.cta_begin[c];
-    __syncthreads();  // the previous virtual CTA's merge is done with shared memory
-    switch (mp.shape[c]) {
-      case 0: walk2_cta<T, multi_shape_vec(0), multi_shape_G(0)>(a, cta, smem, s_row, w_row); break;
-      case 1: walk2_cta<T, multi_shape_vec(1), multi_shape_G(1)>(a, cta, smem, s_row, w_row); break;
-      case 2: walk2_cta<T, multi_shape_vec(2), multi_shape_G(2)>(a, cta, smem, s_row, w_row); break;
-      case 3: walk2_cta<T, multi_shape_vec(3), multi_shape_G(3)>(a, cta, smem, s_row, w_row); break;
-      case 4: walk2_cta<T, multi_shape_vec(4), multi_shape_G(4)>(a, cta, smem, s_row, w_row); break;
-      default: walk2_cta<T, multi_shape_vec(5), multi_shape_G(5)>(a, cta, smem, s_row, w_row); break;
-    }
-  }
-}
-
-// Launch the batched walk (defined in the batch instantiation units).
-template <typename T>
-cudaError_t launch_walk2_multi(const MultiWalkParams& mp, size_t smem, int grid, cudaStream_t s);
-
 // Launchers of the carry fix-up (mttkrp.cu) and of the segment-start search
 // (build.cu), shared with the allocation-free entry point.
 cudaError_t launch_mttkrp_fixup(const int32_t* carry_row, const float* carry,
@@ -704,9 +747,10 @@ cudaError_t launch_mttkrp_fixup(const int32_t* carry_row, const float* carry,
                                 cudaStream_t s);
 cudaError_t launch_segment_starts(const int64_t* nz_ptr, int64_t nfib, int64_t nseg, int64_t seg,
                                   int32_t* seg_fib, cudaStream_t s);
-// Zero bits[(nnz + 31) / 32] and set the bit of the last nonzero of every fiber.
-cudaError_t launch_fiber_end_bits(const int64_t* nz_ptr, int64_t nfib, int64_t nnz, uint32_t* bits,
-                                  cudaStream_t s);
+// Zero end_bits and row_bits ((nnz + 31) / 32 words each) and set the bits of
+// the last nonzero of every fiber and of the first nonzero of every row.
+cudaError_t launch_walk_bits(const int64_t* nz_ptr, const int32_t* fiber_row, int64_t nfib, int64_t nnz,
+                             uint32_t* end_bits, uint32_t* row_bits, cudaStream_t s);
 
 // Launch one walk configuration (defined in the instantiation units).
 template <typename T>
