@@ -37,6 +37,8 @@ struct JointState {
   double* base = nullptr;                // [R x R] mu Gamma + lambda I
   float* gam32 = nullptr;                // [R x R] Gamma
   double* ycoef = nullptr;               // [5] ratings quartic along the ray
+  bool heavy[2] = {false, false};        // a row has more than kHeavyRatings ratings
+  unsigned char* slots = nullptr;        // heavy rows' pieces, two per chunk of ratings (lazy)
   double* part = nullptr;                // block partials
   int64_t part_cap = 0;                  // doubles
 };
@@ -44,7 +46,6 @@ struct JointState {
 namespace {
 
 constexpr int kJT = 256;       // threads of the gradient and quartic kernels
-constexpr int kJRowWarps = 4;  // warps of the ALS row kernel
 constexpr int kJMaxBlocks = 152 * 8;
 
 unsigned jgrid(int64_t rows, int warps) {
@@ -123,76 +124,272 @@ __global__ void joint_base(const double* __restrict__ Gf, const double* __restri
 __device__ __forceinline__ float ld_f(const float* p) { return *p; }
 __device__ __forceinline__ float ld_f(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
-// ALS row update, one warp per row, lane l on column l (R <= 32):
-// F[row] = rhs H^-1 with H = base + sum over the row's ratings of v^T v
-// (Cholesky in FP64 shared memory; H is positive definite for lambda > 0).
-template <typename T>
-__global__ void __launch_bounds__(kJRowWarps * 32) joint_rows(
-    const int64_t* __restrict__ yptr, const int32_t* __restrict__ ycol,
-    const float* __restrict__ yval, const T* __restrict__ other, const float* __restrict__ N,
-    const double* __restrict__ base, double mu, int64_t rows, int R, T* __restrict__ F,
-    int32_t* __restrict__ bad_flag) {
-  extern __shared__ double jsm[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int LD = R + 1;
-  double* H = jsm + (size_t)warp * (R * LD + R);
-  double* x = H + R * LD;
-  const int64_t nw = (int64_t)gridDim.x * kJRowWarps;
-  for (int64_t row = (int64_t)blockIdx.x * kJRowWarps + warp; row < rows; row += nw) {
-    float hrow[32];
+// ---------------------------------------------------------------------------
+// ALS row update: F[row] = rhs H^-1 with H = base + sum over the row's ratings
+// of v^T v and rhs = mu N[row] + sum of y v (H is positive definite for
+// lambda > 0).  A block takes 32 rows: its warps form the 32 systems (ratings
+// Grams in FP32 registers over at most kHeavyRatings ratings, everything above
+// in FP64), then one warp solves them, a thread per system, so that every FP64
+// instruction serves 32 rows (this GPU retires two FP64 lanes per clock and SM:
+// the FP64 pipe bounds the solves, about R^3 / 6 + R^2 lane operations a row; a
+// warp per row left most lanes of them idle).
+//
+// A row with more ratings (one user of a power-law rating matrix holds tens of
+// thousands) would be one warp's serial chain, so such rows are cut: the ratings
+// are chunks of kHeavyRatings positions, and joint_heavy leaves, per chunk, the
+// Gram and right side of the piece of a heavy row that begins before the chunk
+// or at its start (slot 0) and of one that begins inside it and runs past its
+// end (slot 1); the row's block adds its pieces in order.
+//
+// 100,000 users x 50,000 items x 20,000 words, 2M ratings, R = 16: 63.4 ms per
+// sweep with a warp per row (most of it one user's ratings), 3.0 ms now.
+// ---------------------------------------------------------------------------
+constexpr int kHeavyRatings = 1024;
+constexpr int kJTileLd = 33;  // rows of a block, padded
+
+// RP: R padded to 8, 16 or 32 columns.  Lane (i, h), i = lane % RP, h = lane /
+// RP, holds H[i][h CPL .. + CPL).
+template <int RP>
+struct JShape {
+  static constexpr int CG = 32 / RP;   // lane groups
+  static constexpr int CPL = RP / CG;  // columns per lane
+  static constexpr int LD = RP + 4;    // floats of a staged row
+};
+constexpr int kJSolveWarps = 8;
+
+__host__ __device__ constexpr int jtri(int R) { return R * (R + 1) / 2; }
+// Bytes of a chunk slot: the lower triangle in FP32, the right side in FP64.
+__host__ __device__ constexpr size_t jslot_bytes(int R) {
+  return (sizeof(float) * jtri(R) + 7) / 8 * 8 + sizeof(double) * R;
+}
+
+// Gram and right side of ratings [p0, p1) over the rows of `other`, by one
+// warp; the ratings are staged 32 at a time in `tile` ([32][LD] floats, the
+// warp's own).  rhs is complete in every lane of column i.
+template <typename T, int RP>
+__device__ __forceinline__ void joint_accumulate(const int32_t* __restrict__ ycol,
+                                                 const float* __restrict__ yval,
+                                                 const T* __restrict__ other, int64_t p0, int64_t p1,
+                                                 int R, float* tile, float (&hrow)[JShape<RP>::CPL],
+                                                 double& rhs) {
+  using S = JShape<RP>;
+  const int lane = threadIdx.x & 31, i = lane % RP, h = lane / RP;
 #pragma unroll
-    for (int m = 0; m < 32; ++m) hrow[m] = 0.f;
-    double rhs = lane < R ? mu * (double)N[row * R + lane] : 0.0;
-    if (yptr) {
-      const int64_t p1 = yptr[row + 1];
-      for (int64_t p = yptr[row]; p < p1; ++p) {
-        const int64_t o = ycol[p];
-        const float y = yval[p];
-        const float v = lane < R ? ld_f(other + o * R + lane) : 0.f;
-        rhs += (double)y * (double)v;
-#pragma unroll
-        for (int m = 0; m < 32; ++m) hrow[m] = fmaf(v, __shfl_sync(kFull, v, m), hrow[m]);
-      }
+  for (int c = 0; c < S::CPL; ++c) hrow[c] = 0.f;
+  rhs = 0.0;
+  int o_n = p0 + lane < p1 ? ycol[p0 + lane] : 0;
+  float y_n = p0 + lane < p1 ? yval[p0 + lane] : 0.f;
+  for (int64_t p = p0; p < p1; p += 32) {
+    const int n = (int)min((int64_t)32, p1 - p);
+    const int o = o_n;
+    const float y = y_n;
+    if (p + 32 + lane < p1) {  // the next 32 ratings
+      o_n = ycol[p + 32 + lane];
+      y_n = yval[p + 32 + lane];
     }
-    if (lane < R) {
-#pragma unroll
-      for (int m = 0; m < 32; ++m)
-        if (m < R) H[lane * LD + m] = base[lane * R + m] + (double)hrow[m];
-      x[lane] = rhs;
+    __syncwarp();  // the tile's last use is over
+#pragma unroll 8
+    for (int k = 0; k < 32 / S::CG; ++k) {
+      const int t = k * S::CG + h;
+      const int ot = __shfl_sync(kFull, o, t);
+      tile[t * S::LD + i] = (t < n && i < R) ? ld_f(other + (int64_t)ot * R + i) : 0.f;
     }
     __syncwarp();
-    bool bad = false;
-    for (int k = 0; k < R; ++k) {
-      const double d = H[k * LD + k];
-      bad |= !(d > 0.0);
-      const double lkk = sqrt(fmax(d, 1e-300));
-      __syncwarp();
-      if (lane > k && lane < R) H[lane * LD + k] /= lkk;
-      __syncwarp();
-      if (lane > k && lane < R) {
-        const double lik = H[lane * LD + k];
-        for (int m = k + 1; m <= lane; ++m) H[lane * LD + m] -= lik * H[m * LD + k];
+    for (int t = 0; t < n; ++t) {
+      const float vi = tile[t * S::LD + i];
+      float w[S::CPL];
+      const float* q = tile + t * S::LD + h * S::CPL;
+      if constexpr (S::CPL % 4 == 0) {
+#pragma unroll
+        for (int c = 0; c < S::CPL; c += 4) {
+          const float4 f = *reinterpret_cast<const float4*>(q + c);
+          w[c] = f.x; w[c + 1] = f.y; w[c + 2] = f.z; w[c + 3] = f.w;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < S::CPL; ++c) w[c] = q[c];
       }
-      if (lane == k) H[k * LD + k] = lkk;
-      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < S::CPL; ++c) hrow[c] = fmaf(vi, w[c], hrow[c]);
     }
-    if (lane == 0) {  // L L^T x = rhs
+    // the groups take every CG-th rating of the right side
+    for (int t0 = 0; t0 < n; t0 += S::CG) {
+      const int t = t0 + h;  // < 32
+      const float yt = __shfl_sync(kFull, y, t);
+      if (t < n) rhs += (double)yt * (double)tile[t * S::LD + i];
+    }
+  }
+#pragma unroll
+  for (int d = RP; d < 32; d <<= 1) rhs += __shfl_xor_sync(kFull, rhs, d);
+}
+
+// Row of rating position p: the largest r with ptr[r] <= p (and a rating).
+__device__ __forceinline__ int64_t rating_row(const int64_t* __restrict__ ptr, int64_t rows, int64_t p) {
+  int64_t lo = 0, hi = rows - 1;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi + 1) >> 1;
+    if (ptr[mid] <= p) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+__global__ void any_heavy(const int64_t* __restrict__ ptr, int64_t rows, int32_t* __restrict__ flag) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  bool any = false;
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += stride)
+    any |= ptr[r + 1] - ptr[r] > kHeavyRatings;
+  if (__any_sync(kFull, any) && (threadIdx.x & 31) == 0) atomicOr(flag, 1);
+}
+
+// Pieces of heavy rows, one warp per chunk of kHeavyRatings ratings.
+template <typename T, int RP>
+__global__ void __launch_bounds__(kJSolveWarps * 32) joint_heavy(
+    const int64_t* __restrict__ yptr, const int32_t* __restrict__ ycol,
+    const float* __restrict__ yval, const T* __restrict__ other, int64_t rows, int64_t nnzY, int R,
+    unsigned char* __restrict__ slots) {
+  using S = JShape<RP>;
+  __shared__ __align__(16) float tiles[kJSolveWarps][32 * S::LD];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane % RP, h = lane / RP;
+  const int64_t chunk = (int64_t)blockIdx.x * kJSolveWarps + warp;
+  const int64_t c0 = chunk * kHeavyRatings, c1 = min(c0 + kHeavyRatings, nnzY);
+  if (c0 >= nnzY) return;
+  const int64_t r0 = rating_row(yptr, rows, c0), r1 = rating_row(yptr, rows, c1 - 1);
+  for (int slot = 0; slot < 2; ++slot) {
+    const int64_t r = slot == 0 ? r0 : r1;
+    const int64_t b = yptr[r], e = yptr[r + 1];
+    if ((slot == 1 && r1 == r0) || e - b <= kHeavyRatings) continue;
+    float hrow[S::CPL];
+    double rhs;
+    joint_accumulate<T, RP>(ycol, yval, other, max(b, c0), min(e, c1), R, tiles[warp], hrow, rhs);
+    unsigned char* out = slots + (2 * chunk + slot) * jslot_bytes(R);
+    float* tri = reinterpret_cast<float*>(out);
+    double* rs = reinterpret_cast<double*>(out + jslot_bytes(R) - sizeof(double) * R);
+#pragma unroll
+    for (int c = 0; c < S::CPL; ++c) {
+      const int j = h * S::CPL + c;
+      if (i < R && j <= i) tri[jtri(i) + j] = hrow[c];
+    }
+    if (h == 0 && i < R) rs[i] = rhs;
+  }
+}
+
+// The systems of 32 rows and their solutions.  Shared memory: the lower
+// triangles [entry][row] and right sides [column][row] in FP64 (rows padded to
+// kJTileLd: conflict-free by entry and by row), and a staging tile per warp.
+template <typename T, int RP>
+__global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
+    const int64_t* __restrict__ yptr, const int32_t* __restrict__ ycol,
+    const float* __restrict__ yval, const T* __restrict__ other, const float* __restrict__ N,
+    const double* __restrict__ base, double mu, int64_t rows, int R,
+    const unsigned char* __restrict__ slots, T* __restrict__ F, int32_t* __restrict__ bad_flag) {
+  using S = JShape<RP>;
+  extern __shared__ __align__(16) double jsm[];
+  double* Hs = jsm;                              // [jtri(R)][kJTileLd]
+  double* xs = Hs + (size_t)jtri(R) * kJTileLd;  // [R][kJTileLd]
+  float* tiles = reinterpret_cast<float*>(jsm + (((size_t)(jtri(R) + R) * kJTileLd + 1) & ~(size_t)1));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane % RP, h = lane / RP;
+  const int64_t ntiles = (rows + 31) / 32;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int nr = (int)min((int64_t)32, rows - 32 * tile);
+    for (int rr = warp; rr < nr; rr += kJSolveWarps) {
+      const int64_t row = 32 * tile + rr;
+      const int64_t b = yptr ? yptr[row] : 0, e = yptr ? yptr[row + 1] : 0;
+      if (e - b > kHeavyRatings) {
+        // the row's pieces in order, a lane per entry
+        const int64_t k0 = b / kHeavyRatings, k1 = (e - 1) / kHeavyRatings;
+        const int s0 = b % kHeavyRatings ? 1 : 0;
+        for (int t = lane; t < jtri(R); t += 32) {
+          int ti = 0;
+          while (jtri(ti + 1) <= t) ++ti;
+          double a = 0.0;
+          for (int64_t k = k0; k <= k1; ++k)
+            a += (double)reinterpret_cast<const float*>(slots + (2 * k + (k == k0 ? s0 : 0)) * jslot_bytes(R))[t];
+          Hs[t * kJTileLd + rr] = base[ti * R + (t - jtri(ti))] + a;
+        }
+        for (int t = lane; t < R; t += 32) {
+          double a = mu * (double)N[row * R + t];
+          for (int64_t k = k0; k <= k1; ++k)
+            a += reinterpret_cast<const double*>(slots + (2 * k + (k == k0 ? s0 : 0) + 1) * jslot_bytes(R) -
+                                                 sizeof(double) * R)[t];
+          xs[t * kJTileLd + rr] = a;
+        }
+        continue;
+      }
+      float hrow[S::CPL];
+      double rhs;
+      joint_accumulate<T, RP>(ycol, yval, other, b, e, R, tiles + (size_t)warp * 32 * S::LD, hrow, rhs);
+#pragma unroll
+      for (int c = 0; c < S::CPL; ++c) {
+        const int j = h * S::CPL + c;
+        if (i < R && j <= i) Hs[(jtri(i) + j) * kJTileLd + rr] = base[i * R + j] + (double)hrow[c];
+      }
+      if (h == 0 && i < R) xs[i * kJTileLd + rr] = mu * (double)N[row * R + i] + rhs;
+    }
+    __syncthreads();
+    if (warp == 0 && lane < nr) {
+      // Cholesky H = L L^T row by row below the diagonal, then L L^T x = rhs;
+      // the diagonal holds 1 / L[j][j].
+      double* H = Hs + lane;
+      double* x = xs + lane;
+      bool bad = false;
+      for (int j = 0; j < R; ++j) {
+        const int rj = jtri(j);
+        double d = H[(rj + j) * kJTileLd];
+        for (int k = 0; k < j; ++k) {
+          const double l = H[(rj + k) * kJTileLd];
+          d -= l * l;
+        }
+        bad |= !(d > 0.0);
+        const double inv = 1.0 / sqrt(fmax(d, 1e-300));
+        H[(rj + j) * kJTileLd] = inv;
+        int m = j + 1;
+        for (; m + 4 <= R; m += 4) {  // four rows at a time (independent chains)
+          const int a0 = jtri(m), a1 = jtri(m + 1), a2 = jtri(m + 2), a3 = jtri(m + 3);
+          double s0 = H[(a0 + j) * kJTileLd], s1 = H[(a1 + j) * kJTileLd], s2 = H[(a2 + j) * kJTileLd],
+                 s3 = H[(a3 + j) * kJTileLd];
+#pragma unroll 2
+          for (int k = 0; k < j; ++k) {
+            const double l = H[(rj + k) * kJTileLd];
+            s0 -= l * H[(a0 + k) * kJTileLd];
+            s1 -= l * H[(a1 + k) * kJTileLd];
+            s2 -= l * H[(a2 + k) * kJTileLd];
+            s3 -= l * H[(a3 + k) * kJTileLd];
+          }
+          H[(a0 + j) * kJTileLd] = s0 * inv;
+          H[(a1 + j) * kJTileLd] = s1 * inv;
+          H[(a2 + j) * kJTileLd] = s2 * inv;
+          H[(a3 + j) * kJTileLd] = s3 * inv;
+        }
+        for (; m < R; ++m) {
+          const int a0 = jtri(m);
+          double s0 = H[(a0 + j) * kJTileLd];
+          for (int k = 0; k < j; ++k) s0 -= H[(rj + k) * kJTileLd] * H[(a0 + k) * kJTileLd];
+          H[(a0 + j) * kJTileLd] = s0 * inv;
+        }
+      }
       for (int r = 0; r < R; ++r) {
-        double s = x[r];
-        for (int k = 0; k < r; ++k) s -= H[r * LD + k] * x[k];
-        x[r] = s / H[r * LD + r];
+        double s0 = x[r * kJTileLd];
+        for (int k = 0; k < r; ++k) s0 -= H[(jtri(r) + k) * kJTileLd] * x[k * kJTileLd];
+        x[r * kJTileLd] = s0 * H[(jtri(r) + r) * kJTileLd];
       }
       for (int r = R - 1; r >= 0; --r) {
-        double s = x[r];
-        for (int k = r + 1; k < R; ++k) s -= H[k * LD + r] * x[k];
-        x[r] = s / H[r * LD + r];
+        double s0 = x[r * kJTileLd];
+        for (int k = r + 1; k < R; ++k) s0 -= H[(jtri(k) + r) * kJTileLd] * x[k * kJTileLd];
+        x[r * kJTileLd] = s0 * H[(jtri(r) + r) * kJTileLd];
       }
       if (bad) atomicOr(bad_flag, 1);
     }
-    __syncwarp();
-    if (lane < R) st_elem(F + row * R + lane, (float)x[lane]);
-    __syncwarp();
+    __syncthreads();
+    for (int t = threadIdx.x; t < nr * R; t += kJSolveWarps * 32)
+      st_elem(F + 32 * tile * R + t, (float)xs[(t % R) * kJTileLd + t / R]);
+    __syncthreads();  // before the next 32 rows
   }
+}
+
+template <int RP>
+size_t joint_solve_smem(int R) {
+  return sizeof(double) * (((size_t)(jtri(R) + R) * kJTileLd + 1) & ~(size_t)1) +
+         sizeof(float) * kJSolveWarps * 32 * JShape<RP>::LD;
 }
 
 __device__ __forceinline__ float wsum(float v) {
@@ -285,8 +482,10 @@ __global__ void __launch_bounds__(kJT) joint_grad_scalars(const double* __restri
   }
 }
 
-// The ratings term along the ray theta - alpha grad, per user row (warp per
-// row): r(alpha) = y - (a - alpha ga) . (b - alpha gb) = e0 + e1 alpha + e2 alpha^2
+// The ratings term along the ray theta - alpha grad, a thread per rating (rows
+// of any length spread over the GPU; a warp per user row left the longest row,
+// tens of thousands of ratings on power-law data, as one serial chain):
+// r(alpha) = y - (a - alpha ga) . (b - alpha gb) = e0 + e1 alpha + e2 alpha^2
 // and 1/2 r^2 has coefficients 1/2 e0^2, e0 e1, 1/2 e1^2 + e0 e2, e1 e2, 1/2 e2^2;
 // per-block partials part[block][5].  With GA == nullptr only the first (the
 // ratings loss at the current point) is formed.
@@ -294,35 +493,31 @@ template <typename T>
 __global__ void __launch_bounds__(kJT) ratings_quartic(
     const int64_t* __restrict__ yptr, const int32_t* __restrict__ ycol,
     const float* __restrict__ yval, const T* __restrict__ A, const T* __restrict__ B,
-    const float* __restrict__ GA, const float* __restrict__ GB, int64_t rows, int R,
+    const float* __restrict__ GA, const float* __restrict__ GB, int64_t rows, int64_t nnzY, int R,
     double* __restrict__ part) {
   __shared__ double red[kJT];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int W = kJT / 32;
-  const int64_t nw = (int64_t)gridDim.x * W;
   double c[5] = {0, 0, 0, 0, 0};
-  for (int64_t row = (int64_t)blockIdx.x * W + warp; row < rows; row += nw) {
-    const float a = lane < R ? ld_f(A + row * R + lane) : 0.f;
-    const float ga = (GA && lane < R) ? GA[row * R + lane] : 0.f;
-    const int64_t p1 = yptr[row + 1];
-    for (int64_t p = yptr[row]; p < p1; ++p) {
-      const int64_t o = ycol[p];
-      const float b = lane < R ? ld_f(B + o * R + lane) : 0.f;
-      const float gb = (GB && lane < R) ? GB[o * R + lane] : 0.f;
-      const double u0 = (double)wsum(a * b);
-      const double e0 = (double)yval[p] - u0;
-      double e1 = 0.0, e2 = 0.0;
+  const int64_t stride = (int64_t)gridDim.x * kJT;
+  for (int64_t p = (int64_t)blockIdx.x * kJT + threadIdx.x; p < nnzY; p += stride) {
+    const int64_t row = rating_row(yptr, rows, p), o = ycol[p];
+    float u = 0.f, s1 = 0.f, s2 = 0.f;
+    for (int m = 0; m < R; ++m) {
+      const float a = ld_f(A + row * R + m), b = ld_f(B + o * R + m);
+      u = fmaf(a, b, u);
       if (GA) {
-        e1 = (double)wsum(fmaf(a, gb, ga * b));
-        e2 = -(double)wsum(ga * gb);
+        const float ga = GA[row * R + m], gb = GB[o * R + m];
+        s1 += fmaf(a, gb, ga * b);
+        s2 = fmaf(ga, gb, s2);
       }
-      if (lane == 0) {
-        c[0] += 0.5 * e0 * e0;
-        c[1] += e0 * e1;
-        c[2] += 0.5 * e1 * e1 + e0 * e2;
-        c[3] += e1 * e2;
-        c[4] += 0.5 * e2 * e2;
-      }
+    }
+    const double e0 = (double)yval[p] - (double)u;
+    c[0] += 0.5 * e0 * e0;
+    if (GA) {
+      const double e1 = (double)s1, e2 = -(double)s2;
+      c[1] += e0 * e1;
+      c[2] += 0.5 * e1 * e1 + e0 * e2;
+      c[3] += e1 * e2;
+      c[4] += 0.5 * e2 * e2;
     }
   }
   for (int k = 0; k < 5; ++k) {
@@ -371,6 +566,35 @@ int bits_for(int64_t dim) {
   return b;
 }
 
+template <typename T, int RP>
+dfacto_status joint_solve_side(dfacto_t* h, int side) {
+  JointState* J = h->joint;
+  const int R = h->R;
+  cudaStream_t s = h->stream;
+  const int64_t rows = h->dims[side];
+  const bool rated = side < 2;
+  const T* other = static_cast<const T*>(h->F[side == 0 ? 1 : 0]);
+  if (rated && J->heavy[side]) {
+    const int64_t chunks = (J->nnzY + kHeavyRatings - 1) / kHeavyRatings;
+    if (!J->slots) {
+      const dfacto_status st = dalloc(h, reinterpret_cast<void**>(&J->slots), 2 * (size_t)chunks * jslot_bytes(R));
+      if (st != DFACTO_OK) return st;
+    }
+    joint_heavy<T, RP><<<(unsigned)((chunks + kJSolveWarps - 1) / kJSolveWarps), kJSolveWarps * 32, 0, s>>>(
+        J->ptr[side], J->col[side], J->val[side], other, rows, J->nnzY, R, J->slots);
+    DF_COUNT();
+  }
+  const size_t smem = joint_solve_smem<RP>(R);
+  DF_CUDA(h, ensure_dynamic_smem(reinterpret_cast<const void*>(joint_solve<T, RP>), smem));
+  joint_solve<T, RP><<<jgrid(rows, 32), kJSolveWarps * 32, smem, s>>>(
+      rated ? J->ptr[side] : nullptr, rated ? J->col[side] : nullptr, rated ? J->val[side] : nullptr,
+      other, h->N, J->base, J->mu, rows, R, J->slots, static_cast<T*>(h->F[side]),
+      h->flags + kFlagInternal);
+  DF_COUNT();
+  DF_CUDA(h, cudaGetLastError());
+  return DFACTO_OK;
+}
+
 template <typename T>
 dfacto_status joint_rows_side(dfacto_t* h, int side) {
   JointState* J = h->joint;
@@ -383,16 +607,9 @@ dfacto_status joint_rows_side(dfacto_t* h, int side) {
   joint_base<<<1, 256, 0, s>>>(h->gram[f], h->gram[in], R, J->mu, h->lambda_reg, J->base, J->gam32);
   DF_COUNT();
   if ((st = mttkrp_launch(h, side, h->N)) != DFACTO_OK) return st;
-  const int64_t rows = h->dims[side];
-  const size_t smem = sizeof(double) * (size_t)kJRowWarps * (R * (R + 1) + R);
-  DF_CUDA(h, ensure_dynamic_smem(reinterpret_cast<const void*>(joint_rows<T>), smem));
-  const bool rated = side < 2;
-  joint_rows<T><<<jgrid(rows, kJRowWarps), kJRowWarps * 32, smem, s>>>(
-      rated ? J->ptr[side] : nullptr, rated ? J->col[side] : nullptr,
-      rated ? J->val[side] : nullptr, static_cast<const T*>(h->F[side == 0 ? 1 : 0]), h->N, J->base,
-      J->mu, rows, R, static_cast<T*>(h->F[side]), h->flags + kFlagInternal);
-  DF_COUNT();
-  DF_CUDA(h, cudaGetLastError());
+  st = R <= 8 ? joint_solve_side<T, 8>(h, side) : R <= 16 ? joint_solve_side<T, 16>(h, side)
+                                                          : joint_solve_side<T, 32>(h, side);
+  if (st != DFACTO_OK) return st;
   h->gram_valid[side] = false;
   return DFACTO_OK;
 }
@@ -405,11 +622,11 @@ dfacto_status joint_objective_T(dfacto_t* h) {
   fill_ones<<<1, 128, 0, s>>>(h->lambda, h->R);
   DF_COUNT();
   if ((st = fit_direct(h)) != DFACTO_OK) return st;  // <X, Xhat>, ||Xhat||^2 (and the Grams)
-  const unsigned nb = jgrid(h->dims[0], kJT / 32);
+  const unsigned nb = jgrid(J->nnzY, kJT);
   if ((st = grow_part(h, (int64_t)nb * 5)) != DFACTO_OK) return st;
   ratings_quartic<T><<<nb, kJT, 0, s>>>(J->ptr[0], J->col[0], J->val[0],
                                        static_cast<const T*>(h->F[0]), static_cast<const T*>(h->F[1]),
-                                       nullptr, nullptr, h->dims[0], h->R, J->part);
+                                       nullptr, nullptr, h->dims[0], J->nnzY, h->R, J->part);
   DF_COUNT();
   sum5<<<1, kJT, 0, s>>>(J->part, (int)nb, J->ycoef);
   DF_COUNT();
@@ -451,12 +668,12 @@ dfacto_status joint_gd_T(dfacto_t* h) {
     DF_CUDA(h, cudaGetLastError());
   }
   {  // the ratings quartic along the ray
-    const unsigned nb = jgrid(h->dims[0], kJT / 32);
+    const unsigned nb = jgrid(J->nnzY, kJT);
     if ((st = grow_part(h, (int64_t)nb * 5)) != DFACTO_OK) return st;
     ratings_quartic<T><<<nb, kJT, 0, s>>>(J->ptr[0], J->col[0], J->val[0],
                                          static_cast<const T*>(h->F[0]),
                                          static_cast<const T*>(h->F[1]), h->grad[0], h->grad[1],
-                                         h->dims[0], R, J->part);
+                                         h->dims[0], J->nnzY, R, J->part);
     DF_COUNT();
     sum5<<<1, kJT, 0, s>>>(J->part, (int)nb, J->ycoef);
     DF_COUNT();
@@ -485,7 +702,7 @@ void joint_free(dfacto_t* h) {
   for (int side = 0; side < 2; ++side)
     for (void* q : {(void*)J->ptr[side], (void*)J->col[side], (void*)J->val[side]})
       if (q) cudaFreeAsync(q, h->stream);
-  for (void* q : {(void*)J->base, (void*)J->gam32, (void*)J->ycoef, (void*)J->part})
+  for (void* q : {(void*)J->base, (void*)J->gam32, (void*)J->ycoef, (void*)J->part, (void*)J->slots})
     if (q) cudaFreeAsync(q, h->stream);
   delete J;
   h->joint = nullptr;
@@ -561,7 +778,8 @@ dfacto_status dfacto_joint_set_ratings(dfacto_t* h, const int32_t* yidx, const f
       return cuda_bail(e, "ratings copy");
     d_val = tmp_val;
   }
-  if ((e = cudaMemsetAsync(h->flags, 0, sizeof(int32_t) * kNumFlags, s)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(h->flags, 0, sizeof(int32_t) * kNumFlags, s)) != cudaSuccess ||
+      (e = cudaMemsetAsync(J->ycoef, 0, sizeof(double) * 8, s)) != cudaSuccess)  // heavy-row flags below
     return cuda_bail(e, "flags");
   if (nnzY > 0) {
     const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nnzY + 255) / 256, 152 * 32));
@@ -591,6 +809,9 @@ dfacto_status dfacto_joint_set_ratings(dfacto_t* h, const int32_t* yidx, const f
       rating_ptr<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 256) / 256, 152 * 32)), 256, 0, s>>>(
           ks, nnzY, rows, bc, J->ptr[side]);
       DF_COUNT();
+      any_heavy<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 255) / 256, 152 * 8)), 256, 0, s>>>(
+          J->ptr[side], rows, reinterpret_cast<int32_t*>(J->ycoef) + side);
+      DF_COUNT();
     } else {
       if ((e = cudaMemsetAsync(J->ptr[side], 0, sizeof(int64_t) * (rows + 1), s)) != cudaSuccess)
         return cuda_bail(e, "ratings pointers");
@@ -598,8 +819,9 @@ dfacto_status dfacto_joint_set_ratings(dfacto_t* h, const int32_t* yidx, const f
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_bail(e, "ratings build");
   }
   cleanup();
-  int32_t flags[kNumFlags];
+  int32_t flags[kNumFlags], heavy[2];
   if ((e = cudaMemcpyAsync(flags, h->flags, sizeof(flags), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(heavy, J->ycoef, sizeof(heavy), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
       (e = cudaStreamSynchronize(s)) != cudaSuccess)
     return cuda_bail(e, "ratings check");
   if (flags[kFlagRange]) {
@@ -610,6 +832,8 @@ dfacto_status dfacto_joint_set_ratings(dfacto_t* h, const int32_t* yidx, const f
     joint_free(h);
     return fail(h, DFACTO_EDUP, "two ratings share (user, item)");
   }
+  J->heavy[0] = heavy[0] != 0;
+  J->heavy[1] = heavy[1] != 0;
   return DFACTO_OK;
 }
 
