@@ -131,6 +131,8 @@ cudaError_t convert_from(const S* src, void* dst, int dst_dtype, int64_t n, cuda
 cudaError_t convert(const void* src, int src_dtype, void* dst, int dst_dtype, int64_t n,
                     cudaStream_t s) {
   if (n == 0) return cudaSuccess;
+  if (src_dtype == dst_dtype)
+    return cudaMemcpyAsync(dst, src, n * elem_size(src_dtype), cudaMemcpyDeviceToDevice, s);
   if (src_dtype == DFACTO_F32) return convert_from((const float*)src, dst, dst_dtype, n, s);
   if (src_dtype == DFACTO_BF16) return convert_from((const __nv_bfloat16*)src, dst, dst_dtype, n, s);
   return convert_from((const double*)src, dst, dst_dtype, n, s);
@@ -171,7 +173,7 @@ dfacto_status convert_factor_in(dfacto_t* h, int m, const void* src, int src_dty
   if (!is_device_ptr(src) && src_dtype == h->dtype) {  // same type: one copy into the factor
     DF_CUDA(h, cudaMemcpyAsync(h->F[m], src, n * elem_size(src_dtype), cudaMemcpyHostToDevice, h->stream));
     DF_CUDA(h, cudaStreamSynchronize(h->stream));  // caller may free its host buffer
-    h->gram_valid[m] = false;
+    h->gram_valid[m] = h->pad_valid[m] = false;
     return DFACTO_OK;
   }
   if (!is_device_ptr(src)) {
@@ -183,7 +185,7 @@ dfacto_status convert_factor_in(dfacto_t* h, int m, const void* src, int src_dty
   if (tmp) cudaFreeAsync(tmp, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "factor conversion");
   if (tmp) DF_CUDA(h, cudaStreamSynchronize(h->stream));  // caller may free its host buffer
-  h->gram_valid[m] = false;
+  h->gram_valid[m] = h->pad_valid[m] = false;
   return DFACTO_OK;
 }
 
@@ -258,7 +260,8 @@ void dfacto_destroy(dfacto_t* h) {
   for (void* q : {(void*)h->N, (void*)h->Fh, (void*)h->lambda, (void*)h->inv_lambda, (void*)h->ipart,
                   (void*)h->gd_mats, (void*)h->gd_scratch, (void*)h->W, (void*)h->rr_work, (void*)h->W32, (void*)h->scal,
                   (void*)h->flags, (void*)h->partials, (void*)h->carry, (void*)h->carry_row,
-                  (void*)h->pad_in, (void*)h->pad_f, (void*)h->pad_out, (void*)h->pad_dual,
+                  (void*)h->pad_F[0], (void*)h->pad_F[1], (void*)h->pad_F[2], (void*)h->pad_out,
+                  (void*)h->pad_dual,
                   (void*)h->ls_vals})
     if (q) cudaFreeAsync(q, h->stream);
   delete[] h->host_scal;

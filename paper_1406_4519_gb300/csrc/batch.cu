@@ -752,7 +752,10 @@ dfacto_status dfacto_batch_als_iter(dfacto_batch_t* b, double* fits) {
   if (st != DFACTO_OK) return st;
   bool grams_known = true;
   for (dfacto_t* h : b->jobs)
-    for (int m = 0; m < 3; ++m) grams_known = grams_known && h->gram_valid[m];
+    for (int m = 0; m < 3; ++m) {
+      grams_known = grams_known && h->gram_valid[m];
+      h->pad_valid[m] = false;  // the sweep, launched or replayed, changes every factor
+    }
   if (!grams_known) drop_graph(b);  // factors changed outside the batch
   if (b->opt.use_graph && grams_known && !b->graph_ready) {
     // Capture one sweep.  Every host-side decision the sweep makes (Grams

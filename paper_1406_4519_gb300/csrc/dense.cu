@@ -24,8 +24,6 @@
 
 namespace dfacto {
 
-dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out);
-
 namespace {
 
 constexpr int kT = 256;          // threads of the row-pass and Gram kernels
@@ -192,23 +190,22 @@ __global__ void __launch_bounds__(kT) gram_tiles(const TX* __restrict__ X, const
     }
     __syncthreads();
   }
-  // Combine the row groups of each block in group order, write the partial.
+  // Combine the row groups of each block in group order, write the partial: a
+  // thread per entry.
   double* red = reinterpret_cast<double*>(sm);  // [kT][16] (fits the tile space)
 #pragma unroll
   for (int b = 0; b < BPT; ++b) {
-    const int blk = nblk <= kT ? (int)threadIdx.x % nblk : (int)threadIdx.x + b * kT;
 #pragma unroll
     for (int q = 0; q < 16; ++q) red[threadIdx.x * 16 + q] = acc[b][q];
     __syncthreads();
-    if (owner && grp == 0 && blk < nblk) {
-      const int bi = blk / R4, bj = blk % R4;
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        double t = 0.0;
-        for (int gg = 0; gg < ngrp; ++gg) t += red[(gg * nblk + (nblk <= kT ? blk : (int)threadIdx.x)) * 16 + q];
-        const int a = 4 * bi + q / 4, c = 4 * bj + q % 4;
-        if (a < R && c < R) part[(size_t)blockIdx.x * R * R + a * R + c] = t;
-      }
+    const int owned = nblk <= kT ? nblk : min(kT, nblk - b * kT);  // blocks of this round
+    for (int e = threadIdx.x; e < owned * 16; e += kT) {
+      const int blk = e / 16, q = e % 16, gb = nblk <= kT ? blk : blk + b * kT;
+      const int bi = gb / R4, bj = gb % R4;
+      double t = 0.0;
+      for (int gg = 0; gg < ngrp; ++gg) t += red[(gg * nblk + blk) * 16 + q];
+      const int i = 4 * bi + q / 4, c = 4 * bj + q % 4;
+      if (i < R && c < R) part[(size_t)blockIdx.x * R * R + i * R + c] = t;
     }
     __syncthreads();
   }
@@ -236,60 +233,129 @@ __device__ __forceinline__ void gamma_inverse_body(const double* __restrict__ Gf
   const int tid = threadIdx.x, nt = blockDim.x;
   const int RR = R * R;
   const double eps = 2.220446049250313e-16;
-  for (int e = tid; e < RR; e += nt) {
-    double g = Gf[e] * Gi[e];
-    if (e / R == e % R) g += lambda_reg;
-    A[e] = g;
-  }
-  if (tid == 0) failed = 0;
-  __syncthreads();
-  for (int a = tid; a < R; a += nt) d0[a] = A[a * R + a];
-  __syncthreads();
-  // Right-looking Cholesky, lower triangle.
-  for (int j = 0; j < R; ++j) {
-    if (tid == 0) {
-      const double d = A[j * R + j];
-      if (!(d0[j] > 0.0) || !(d > (double)R * eps * d0[j])) failed = 1;
-      else A[j * R + j] = sqrt(d);
-    }
-    __syncthreads();
-    if (failed) break;
-    const double rjj = 1.0 / A[j * R + j];
-    for (int i = j + 1 + tid; i < R; i += nt) A[i * R + j] *= rjj;
-    __syncthreads();
-    const int m = R - j - 1;
-    for (int e = tid; e < m * m; e += nt) {
-      const int i = j + 1 + e / m, k = j + 1 + e % m;
-      if (k <= i) A[i * R + k] -= A[i * R + j] * A[k * R + j];
-    }
-    __syncthreads();
-  }
-  if (!failed) {
-    // Linv by forward substitution, one column per thread (reciprocal
-    // diagonal in d0).
-    for (int a = tid; a < R; a += nt) d0[a] = 1.0 / A[a * R + a];
-    __syncthreads();
-    for (int c = tid; c < R; c += nt) {
-      for (int i = 0; i < R; ++i) {
-        if (i < c) {
-          B[i * R + c] = 0.0;
-        } else {
-          double s = (i == c) ? 1.0 : 0.0;
-          for (int k = c; k < i; ++k) s -= A[i * R + k] * B[k * R + c];
-          B[i * R + c] = s * d0[i];
+  if (R <= 32) {
+    // Gauss-Jordan in place, entry (i, j) = (tid / 32 + 8 m, tid % 32) in the
+    // registers of its thread, one barrier per pivot; the pivots are Cholesky's
+    // squared (Schur complements of a positive definite matrix, which needs no
+    // pivoting).  An SM retires two FP64 lanes per clock, half a lane per warp
+    // scheduler: a warp alone gets an FP64 instruction done in 64 clocks, so the
+    // R^3 of this form, spread over eight warps with no other phase, beats the
+    // Cholesky factor, its inverse and their product (R = 32: 80 us, 37 now).
+    __shared__ double rowb[2][32], colb[2][32], rinv[2], diag[32];
+    __shared__ int bad[2];  // pivot k failed, by k % 2 (read before it is written again)
+    const int j = tid & 31, i0 = tid >> 5;
+    double x[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int i = i0 + 8 * m;
+      x[m] = 0.0;
+      if (i < R && j < R) {
+        x[m] = Gf[i * R + j] * Gi[i * R + j];
+        if (i == j) {
+          x[m] += lambda_reg;
+          diag[i] = x[m];
         }
       }
     }
     __syncthreads();
-    // W = Linv^T Linv.
-    for (int e = tid; e < RR; e += nt) {
-      const int a = e / R, b = e % R;
-      double s = 0.0;
-      for (int k = max(a, b); k < R; ++k) s += B[k * R + a] * B[k * R + b];
-      W[e] = s;
-      W32[e] = (float)s;
+    auto publish = [&](int k) {  // row k, column k and the reciprocal of pivot k
+      const int buf = k & 1;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int i = i0 + 8 * m;
+        if (i == k) rowb[buf][j] = x[m];
+        if (j == k) colb[buf][i] = x[m];
+        if (i == k && j == k) {
+          bad[buf] = !(diag[k] > 0.0) || !(x[m] > (double)R * eps * diag[k]);
+          rinv[buf] = 1.0 / x[m];
+        }
+      }
+    };
+    publish(0);
+    bool ok = true;
+    for (int k = 0; k < R; ++k) {
+      __syncthreads();
+      const int buf = k & 1;
+      if (bad[buf]) {  // the same for every thread
+        ok = false;
+        break;
+      }
+      const double r = rinv[buf], rk = j == k ? r : rowb[buf][j] * r;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int i = i0 + 8 * m;
+        if (i == k) x[m] = rk;
+        else x[m] = (j == k ? 0.0 : x[m]) - colb[buf][i] * rk;
+      }
+      if (k + 1 < R) publish(k + 1);
     }
-    return;
+    if (ok) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int i = i0 + 8 * m;
+        if (i < R && j < R) {
+          W[i * R + j] = x[m];
+          W32[i * R + j] = (float)x[m];
+        }
+      }
+      return;
+    }
+  } else {
+    for (int e = tid; e < RR; e += nt) {
+      double g = Gf[e] * Gi[e];
+      if (e / R == e % R) g += lambda_reg;
+      A[e] = g;
+    }
+    if (tid == 0) failed = 0;
+    __syncthreads();
+    for (int a = tid; a < R; a += nt) d0[a] = A[a * R + a];
+    __syncthreads();
+    // Right-looking Cholesky, lower triangle.
+    for (int j = 0; j < R; ++j) {
+      if (tid == 0) {
+        const double d = A[j * R + j];
+        if (!(d0[j] > 0.0) || !(d > (double)R * eps * d0[j])) failed = 1;
+        else A[j * R + j] = sqrt(d);
+      }
+      __syncthreads();
+      if (failed) break;
+      const double rjj = 1.0 / A[j * R + j];
+      for (int i = j + 1 + tid; i < R; i += nt) A[i * R + j] *= rjj;
+      __syncthreads();
+      const int m = R - j - 1;
+      for (int e = tid; e < m * m; e += nt) {
+        const int i = j + 1 + e / m, k = j + 1 + e % m;
+        if (k <= i) A[i * R + k] -= A[i * R + j] * A[k * R + j];
+      }
+      __syncthreads();
+    }
+    if (!failed) {
+      // Linv by forward substitution, one column per thread (reciprocal
+      // diagonal in d0).
+      for (int a = tid; a < R; a += nt) d0[a] = 1.0 / A[a * R + a];
+      __syncthreads();
+      for (int c = tid; c < R; c += nt) {
+        for (int i = 0; i < R; ++i) {
+          if (i < c) {
+            B[i * R + c] = 0.0;
+          } else {
+            double s = (i == c) ? 1.0 : 0.0;
+            for (int k = c; k < i; ++k) s -= A[i * R + k] * B[k * R + c];
+            B[i * R + c] = s * d0[i];
+          }
+        }
+      }
+      __syncthreads();
+      // W = Linv^T Linv.
+      for (int e = tid; e < RR; e += nt) {
+        const int a = e / R, b = e % R;
+        double s = 0.0;
+        for (int k = max(a, b); k < R; ++k) s += B[k * R + a] * B[k * R + b];
+        W[e] = s;
+        W32[e] = (float)s;
+      }
+      return;
+    }
   }
   if (tid == 0) atomicOr(singular, 1);
   for (int e = tid; e < RR; e += nt) {
@@ -1132,9 +1198,13 @@ __device__ __forceinline__ void stage_w(const float* __restrict__ W32, int R, fl
 // when NBLK does not divide kT (RT = 12: 28 groups of 9) the last kT % NBLK
 // threads add nothing.
 template <int RT>
+constexpr int row_ld_t() { return RT == 12 ? RT + 8 : RT + 4; }
+template <int RT>
 struct PassShape {
   static constexpr int CW = RT < 16 ? RT : 16;
-  static constexpr int LD = RT + 4;  // tile row stride (16-byte aligned rows)
+  // tile row stride: 16-byte aligned rows that a warp reads a row per lane
+  // without bank conflicts
+  static constexpr int LD = row_ld_t<RT>();
   static constexpr int NB4 = RT / 4, NBLK = NB4 * NB4, NGRP = kT / NBLK;
 };
 
@@ -1146,15 +1216,16 @@ __device__ __forceinline__ void tile_load(const float* __restrict__ M, int64_t t
                                           float* __restrict__ tile) {
   const float* src = M + t0 * R;
   const int total = nt * R;
+  const uint32_t inv = small_inv(R);
   if ((R & 3) == 0) {
     for (int e4 = threadIdx.x; e4 < (total >> 2); e4 += kT) {
       const float4 v = __ldg(reinterpret_cast<const float4*>(src) + e4);
-      const int e = 4 * e4, r = e / R, c = e - r * R;
+      const int e = 4 * e4, r = small_div(e, inv), c = e - r * R;
       *reinterpret_cast<float4*>(tile + r * LD + c) = v;
     }
   } else {
     for (int e = threadIdx.x; e < total; e += kT) {
-      const int r = e / R, c = e - r * R;
+      const int r = small_div(e, inv), c = e - r * R;
       tile[r * LD + c] = __ldg(src + e);
     }
   }
@@ -1169,8 +1240,9 @@ __device__ __forceinline__ void tile_load_async(const float* __restrict__ M, int
                                                 int R, float* __restrict__ tile) {
   const float* src = M + t0 * R;
   const int total4 = (nt * R) >> 2;
+  const uint32_t inv = small_inv(R);
   for (int e4 = threadIdx.x; e4 < total4; e4 += kT) {
-    const int e = 4 * e4, r = e / R, c = e - r * R;
+    const int e = 4 * e4, r = small_div(e, inv), c = e - r * R;
     const unsigned dst = (unsigned)__cvta_generic_to_shared(tile + r * LD + c);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + e) : "memory");
   }
@@ -1195,7 +1267,7 @@ constexpr size_t row_pass_w_floats() {
 // Shared memory of the double-buffered row passes: W and two tiles.
 template <int RT>
 constexpr size_t row_pass_smem() {
-  return sizeof(float) * (row_pass_w_floats<RT>() + 2 * (size_t)kT * (RT + 4));
+  return sizeof(float) * (row_pass_w_floats<RT>() + 2 * (size_t)kT * row_ld_t<RT>());
 }
 
 // Tile t of a row pass in buffer t & 1: for R % 4 == 0 the next tile's copy is
@@ -1233,14 +1305,15 @@ __device__ __forceinline__ void tile_store(const float* __restrict__ tile, int64
                                            float* __restrict__ M) {
   float* dst = M + t0 * R;
   const int total = nt * R;
+  const uint32_t inv = small_inv(R);
   if ((R & 3) == 0) {
     for (int e4 = threadIdx.x; e4 < (total >> 2); e4 += kT) {
-      const int e = 4 * e4, r = e / R, c = e - r * R;
+      const int e = 4 * e4, r = small_div(e, inv), c = e - r * R;
       reinterpret_cast<float4*>(dst)[e4] = *reinterpret_cast<const float4*>(tile + r * LD + c);
     }
   } else {
     for (int e = threadIdx.x; e < total; e += kT) {
-      const int r = e / R, c = e - r * R;
+      const int r = small_div(e, inv), c = e - r * R;
       dst[e] = tile[r * LD + c];
     }
   }
@@ -1250,9 +1323,10 @@ __device__ __forceinline__ void tile_store(const float* __restrict__ tile, int64
                                            __nv_bfloat16* __restrict__ M) {
   __nv_bfloat16* dst = M + t0 * R;
   const int total = nt * R;
+  const uint32_t inv = small_inv(R);
   if ((R & 7) == 0) {
     for (int e8 = threadIdx.x; e8 < (total >> 3); e8 += kT) {
-      const int e = 8 * e8, r = e / R, c = e - r * R;
+      const int e = 8 * e8, r = small_div(e, inv), c = e - r * R;
       const float* q = tile + r * LD + c;
       uint4 w;
       w.x = (__float_as_uint(q[0]) >> 16) | (__float_as_uint(q[1]) & 0xffff0000u);
@@ -1263,7 +1337,7 @@ __device__ __forceinline__ void tile_store(const float* __restrict__ tile, int64
     }
   } else {
     for (int e = threadIdx.x; e < total; e += kT) {
-      const int r = e / R, c = e - r * R;
+      const int r = small_div(e, inv), c = e - r * R;
       st_elem(dst + e, tile[r * LD + c]);
     }
   }
@@ -1444,7 +1518,7 @@ __device__ __forceinline__ void zero_gram(float (&g)[RT / 16][RT / 8][4]) {
 // (N W)[row, c]^2.  Each lane sums the squares of its fragment entries in
 // FP32; lanes are added by shuffles, warps in FP64 in warp order.
 template <int RT>
-__device__ __forceinline__ void colnorm_rows_tc(const float* __restrict__ N,
+__device__ __forceinline__ void colnorm_rows_tc(const float* __restrict__ N, int ldN,
                                                 const float* __restrict__ W32, int64_t rows, int R,
                                                 double* __restrict__ colsq, int vb, int vgrid) {
   constexpr int LD = RT + 4, WS = row_pass_wstride<RT>(), NS = RT / 8;
@@ -1462,12 +1536,12 @@ __device__ __forceinline__ void colnorm_rows_tc(const float* __restrict__ N,
 #pragma unroll
   for (int n = 0; n < NS; ++n) sq[n][0] = sq[n][1] = 0.f;
   __syncthreads();
-  row_pass_prefetch<LD>(N, r0, r1, R, tiles);
+  row_pass_prefetch<LD>(N, r0, r1, ldN, tiles);
   int buf = 0;
   for (int64_t t0 = r0; t0 < r1; t0 += kT, buf ^= 1) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    const float* tile = row_pass_tile<LD>(N, t0, r1, R, tiles, buf);
+    const float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
@@ -1510,11 +1584,11 @@ __device__ __forceinline__ void colnorm_rows_tc(const float* __restrict__ N,
 // eight rows); the tile is then written to F with coalesced stores.  At the
 // end the warps' Grams are added in FP64, in warp order.
 template <typename T, int RT>
-__device__ __forceinline__ void scale_store_rows_tc(const float* __restrict__ N,
+__device__ __forceinline__ void scale_store_rows_tc(const float* __restrict__ N, int ldN,
                                                     const float* __restrict__ W32,
                                                     const float* __restrict__ inv,
                                                     const double* __restrict__ lambda, int64_t rows,
-                                                    int R, T* __restrict__ F,
+                                                    int R, T* __restrict__ F, float* __restrict__ Fpad,
                                                     double* __restrict__ gpart, bool with_ip,
                                                     double* __restrict__ ipart, int vb, int vgrid) {
   constexpr int LD = RT + 4, WS = row_pass_wstride<RT>(), NS = RT / 8, MB = RT / 16;
@@ -1537,12 +1611,12 @@ __device__ __forceinline__ void scale_store_rows_tc(const float* __restrict__ N,
   int64_t r0, r1;
   block_rows(rows, vb, vgrid, r0, r1);
   __syncthreads();
-  row_pass_prefetch<LD>(N, r0, r1, R, tiles);
+  row_pass_prefetch<LD>(N, r0, r1, ldN, tiles);
   int buf = 0;
   for (int64_t t0 = r0; t0 < r1; t0 += kT, buf ^= 1) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    float* tile = row_pass_tile<LD>(N, t0, r1, R, tiles, buf);
+    float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
     float ip32 = 0.f;
 #pragma unroll
@@ -1568,6 +1642,7 @@ __device__ __forceinline__ void scale_store_rows_tc(const float* __restrict__ N,
     warp_gram_acc<RT>(tile, tile, 32 * warp, g);
     __syncthreads();
     tile_store<LD>(tile, t0, nt, R, F);
+    if (Fpad) tile_store<LD>(tile, t0, nt, ldN, Fpad);  // columns R .. ldN-1 of the tile are zero
   }
   if (with_ip) {
     const double t = block_sum(ip, red);
@@ -1576,21 +1651,50 @@ __device__ __forceinline__ void scale_store_rows_tc(const float* __restrict__ N,
   fold_warp_grams<RT>(g, tiles, R, gpart, vb);  // NW x RT x RT floats <= 2 kT LD floats
 }
 
+// Sum the per-thread 4 x 4 block partials a32 of the groups of each block in
+// FP64 (P threads per entry, each its share of the groups in order, then the
+// shares) through `scratch` (16 kT floats), and store block vb's R x R partial
+// at gpart[vb][R*R].
+template <int RT>
+__device__ __forceinline__ void store_gram_partial(const float (&a32)[16], float* scratch, int R,
+                                                   double* __restrict__ gpart, int vb) {
+  using PS = PassShape<RT>;
+  constexpr int NB4 = PS::NB4, NBLK = PS::NBLK, NGRP = PS::NGRP;
+  constexpr int P = kT / (NBLK * 16) >= 4 ? 4 : 1;
+  static_assert(2 * kT * PS::LD >= 16 * kT && NGRP % P == 0, "scratch");
+#pragma unroll
+  for (int q = 0; q < 16; ++q) scratch[q * kT + threadIdx.x] = a32[q];
+  __syncthreads();
+  for (int e0 = 0; e0 < NBLK * 16; e0 += kT / P) {
+    const int e = e0 + (int)threadIdx.x / P, part = threadIdx.x % P;
+    const int blk = e / 16, q = e % 16;
+    double t = 0.0;
+    if (e < NBLK * 16)
+      for (int gg = part * (NGRP / P); gg < (part + 1) * (NGRP / P); ++gg)
+        t += (double)scratch[q * kT + gg * NBLK + blk];
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
+    const int a = 4 * (blk / NB4) + q / 4, c = 4 * (blk % NB4) + q % 4;
+    if (e < NBLK * 16 && part == 0 && a < R && c < R) gpart[(size_t)vb * R * R + a * R + c] = t;
+  }
+  __syncthreads();
+}
+
 // Pass 1: colsq[vb][c] = sum over the block's rows of (N W)[row, c]^2.  A tile
 // of kT rows is loaded into shared memory with coalesced loads; thread t then
 // takes row t of the tile.  Each thread sums its rows in FP32; the block adds
 // the threads in FP64, in thread order.
 template <int RT>
-__device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N,
+__device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N, int ldN,
                                                   const float* __restrict__ W32, int64_t rows, int R,
                                                   double* __restrict__ colsq, int vb, int vgrid) {
   if constexpr (row_pass_tc<RT>()) {
-    colnorm_rows_tc<RT>(N, W32, rows, R, colsq, vb, vgrid);
+    colnorm_rows_tc<RT>(N, ldN, W32, rows, R, colsq, vb, vgrid);
     return;
   }
   using PS = PassShape<RT>;
   constexpr int CW = PS::CW, LD = PS::LD;
-  static_assert(LD >= RT + 1, "the tile doubles as the FP64 reduction area");
+  static_assert(2 * LD * kT >= kT * (RT + 1) + 520, "the tiles double as the reduction area");
   extern __shared__ __align__(16) float row_smem[];  // row_pass_smem<RT>() bytes
   float* Ws = row_smem;
   float* tiles = row_smem + row_pass_w_floats<RT>();
@@ -1602,12 +1706,12 @@ __device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N,
 #pragma unroll
   for (int c = 0; c < RT; ++c) sq[c] = 0.f;
   __syncthreads();
-  row_pass_prefetch<LD>(N, r0, r1, R, tiles);
+  row_pass_prefetch<LD>(N, r0, r1, ldN, tiles);
   int buf = 0;
   for (int64_t t0 = r0; t0 < r1; t0 += kT, buf ^= 1) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    const float* tile = row_pass_tile<LD>(N, t0, r1, R, tiles, buf);
+    const float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
     if ((int)threadIdx.x < nt) {
       float n[RT];
@@ -1625,15 +1729,25 @@ __device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N,
       }
     }
   }
+  // The threads' sums in FP64: sixteen threads in order per (column, part), then
+  // the parts in order.
   __syncthreads();
+  static_assert(row_pass_tc<RT>() || (RT <= 16 && kT == 256), "a column per lane of sixteen");
   float* red = tiles;  // [kT][RT + 1]
+  double* parts = reinterpret_cast<double*>(tiles + (size_t)kT * (RT + 1) + (kT * (RT + 1)) % 2);  // [16][16]
 #pragma unroll
   for (int c = 0; c < RT; ++c) red[threadIdx.x * (RT + 1) + c] = sq[c];
   __syncthreads();
+  const int pc = threadIdx.x % 16, pp = threadIdx.x / 16;
+  double t = 0.0;
+  if (pc < R)
+    for (int i = 0; i < 16; ++i) t += (double)red[(pp * 16 + i) * (RT + 1) + pc];
+  parts[pp * 16 + pc] = t;
+  __syncthreads();
   for (int c = threadIdx.x; c < R; c += kT) {
-    double t = 0.0;
-    for (int i = 0; i < kT; ++i) t += (double)red[i * (RT + 1) + c];
-    colsq[(size_t)vb * R + c] = t;
+    double a = 0.0;
+    for (int p = 0; p < 16; ++p) a += parts[p * 16 + c];
+    colsq[(size_t)vb * R + c] = a;
   }
 }
 
@@ -1646,15 +1760,15 @@ __device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N,
 // ipart[vb] = sum lambda_c F_stored[row, c] N[row, c] (the fit's inner
 // product after the last mode).
 template <typename T, int RT>
-__device__ __forceinline__ void scale_store_rows_body(const float* __restrict__ N,
+__device__ __forceinline__ void scale_store_rows_body(const float* __restrict__ N, int ldN,
                                                       const float* __restrict__ W32,
                                                       const float* __restrict__ inv,
                                                       const double* __restrict__ lambda, int64_t rows,
-                                                      int R, T* __restrict__ F,
+                                                      int R, T* __restrict__ F, float* __restrict__ Fpad,
                                                       double* __restrict__ gpart, bool with_ip,
                                                       double* __restrict__ ipart, int vb, int vgrid) {
   if constexpr (row_pass_tc<RT>()) {
-    scale_store_rows_tc<T, RT>(N, W32, inv, lambda, rows, R, F, gpart, with_ip, ipart, vb, vgrid);
+    scale_store_rows_tc<T, RT>(N, ldN, W32, inv, lambda, rows, R, F, Fpad, gpart, with_ip, ipart, vb, vgrid);
     return;
   }
   using PS = PassShape<RT>;
@@ -1679,12 +1793,12 @@ __device__ __forceinline__ void scale_store_rows_body(const float* __restrict__ 
   int64_t r0, r1;
   block_rows(rows, vb, vgrid, r0, r1);
   __syncthreads();
-  row_pass_prefetch<LD>(N, r0, r1, R, tiles);
+  row_pass_prefetch<LD>(N, r0, r1, ldN, tiles);
   int buf = 0;
   for (int64_t t0 = r0; t0 < r1; t0 += kT, buf ^= 1) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    float* tile = row_pass_tile<LD>(N, t0, r1, R, tiles, buf);
+    float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
     float ip32 = 0.f;
     float* trow = tile + threadIdx.x * LD;
@@ -1720,6 +1834,7 @@ __device__ __forceinline__ void scale_store_rows_body(const float* __restrict__ 
     ip += (double)ip32;
     __syncthreads();
     tile_store<LD>(tile, t0, nt, R, F);
+    if (Fpad) tile_store<LD>(tile, t0, nt, ldN, Fpad);  // columns R .. ldN-1 of the tile are zero
     for (int i = grp; grp < NGRP && i < nt; i += NGRP) {
       const float4 xv = *reinterpret_cast<const float4*>(tile + i * LD + 4 * bi);
       const float4 yv = *reinterpret_cast<const float4*>(tile + i * LD + 4 * bj);
@@ -1734,26 +1849,8 @@ __device__ __forceinline__ void scale_store_rows_body(const float* __restrict__ 
     const double t = block_sum(ip, red);
     if (threadIdx.x == 0) ipart[vb] = t;
   }
-  // Add the groups of each block in group order, four entries at a time
-  // through the tile ([kT][4] doubles = 8 KB <= the tile's kT * LD floats).
   __syncthreads();
-  double* rsm = reinterpret_cast<double*>(tiles);
-  for (int q0 = 0; q0 < 16; q0 += 4) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) rsm[threadIdx.x * 4 + q] = (double)a32[q0 + q];
-    __syncthreads();
-    if (grp == 0) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double t = 0.0;
-        for (int gg = 0; gg < NGRP; ++gg) t += rsm[(gg * NBLK + blk) * 4 + q];
-        const int e = q0 + q;
-        const int a = 4 * bi + e / 4, c = 4 * bj + e % 4;
-        if (a < R && c < R) gpart[(size_t)vb * R * R + a * R + c] = t;
-      }
-    }
-    __syncthreads();
-  }
+  store_gram_partial<RT>(a32, tiles, R, gpart, vb);
 }
 
 // Tile rows of a factor in storage type T (BF16 widened), coalesced 16-byte
@@ -1768,47 +1865,20 @@ __device__ __forceinline__ void tile_load_T(const __nv_bfloat16* __restrict__ M,
                                             int R, float* __restrict__ tile) {
   const __nv_bfloat16* src = M + t0 * R;
   const int total = nt * R;
+  const uint32_t inv = small_inv(R);
   if ((R & 7) == 0) {
     for (int e8 = threadIdx.x; e8 < (total >> 3); e8 += kT) {
       const uint4 w = __ldg(reinterpret_cast<const uint4*>(src) + e8);
-      const int e = 8 * e8, r = e / R, c = e - r * R;
+      const int e = 8 * e8, r = small_div(e, inv), c = e - r * R;
       float* q = tile + r * LD + c;
       q[0] = bf16_lo(w.x); q[1] = bf16_hi(w.x); q[2] = bf16_lo(w.y); q[3] = bf16_hi(w.y);
       q[4] = bf16_lo(w.z); q[5] = bf16_hi(w.z); q[6] = bf16_lo(w.w); q[7] = bf16_hi(w.w);
     }
   } else {
     for (int e = threadIdx.x; e < total; e += kT) {
-      const int r = e / R, c = e - r * R;
+      const int r = small_div(e, inv), c = e - r * R;
       tile[r * LD + c] = ld_elem(src + e);
     }
-  }
-}
-
-// Sum the per-thread 4 x 4 block partials a32 of the groups of each block in
-// group order (FP64, four entries at a time through `scratch`, >= kT * 4
-// doubles) and store block vb's R x R partial at gpart[vb][R*R].
-template <int RT>
-__device__ __forceinline__ void store_gram_partial(const float (&a32)[16], double* scratch, int R,
-                                                   double* __restrict__ gpart, int vb) {
-  using PS = PassShape<RT>;
-  constexpr int NB4 = PS::NB4, NBLK = PS::NBLK, NGRP = PS::NGRP;
-  const int blk = threadIdx.x % NBLK, grp = threadIdx.x / NBLK;
-  const int bi = blk / NB4, bj = blk % NB4;
-  for (int q0 = 0; q0 < 16; q0 += 4) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) scratch[threadIdx.x * 4 + q] = (double)a32[q0 + q];
-    __syncthreads();
-    if (grp == 0) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double t = 0.0;
-        for (int gg = 0; gg < NGRP; ++gg) t += scratch[(gg * NBLK + blk) * 4 + q];
-        const int e = q0 + q;
-        const int a = 4 * bi + e / 4, c = 4 * bj + e % 4;
-        if (a < R && c < R) gpart[(size_t)vb * R * R + a * R + c] = t;
-      }
-    }
-    __syncthreads();
   }
 }
 
@@ -1827,7 +1897,7 @@ __device__ __forceinline__ void store_gram_partial(const float (&a32)[16], doubl
 // partials are added in FP64 in warp order.  Dynamic shared memory: Gamma
 // split into heads and tails, and two tiles.
 template <typename T, int RT>
-__device__ __forceinline__ void gd_rows_tc(const float* __restrict__ N, const T* __restrict__ F,
+__device__ __forceinline__ void gd_rows_tc(const float* __restrict__ N, int ldN, const T* __restrict__ F,
                                            const float* __restrict__ Gam32, int64_t rows, int R,
                                            float* __restrict__ grad, double* __restrict__ gpart_gg,
                                            double* __restrict__ gpart_fg,
@@ -1853,7 +1923,7 @@ __device__ __forceinline__ void gd_rows_tc(const float* __restrict__ N, const T*
   for (int64_t t0 = r0; t0 < r1; t0 += kT) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    tile_load<LD>(N, t0, nt, R, tN);
+    tile_load<LD>(N, t0, nt, ldN, tN);
     tile_load_T<LD>(F, t0, nt, R, tF);
     __syncthreads();
     if ((int)threadIdx.x >= nt) {  // rows past the tile's end add nothing
@@ -1898,14 +1968,14 @@ __device__ __forceinline__ void gd_rows_tc(const float* __restrict__ N, const T*
 }
 
 template <typename T, int RT>
-__global__ void __launch_bounds__(kT, 2) gd_rows(const float* __restrict__ N, const T* __restrict__ F,
+__global__ void __launch_bounds__(kT, 2) gd_rows(const float* __restrict__ N, int ldN, const T* __restrict__ F,
                                                  const float* __restrict__ Gam32, int64_t rows, int R,
                                                  float* __restrict__ grad,
                                                  double* __restrict__ gpart_gg,
                                                  double* __restrict__ gpart_fg,
                                                  double* __restrict__ spart) {
   if constexpr (row_pass_tc<RT>()) {
-    gd_rows_tc<T, RT>(N, F, Gam32, rows, R, grad, gpart_gg, gpart_fg, spart);
+    gd_rows_tc<T, RT>(N, ldN, F, Gam32, rows, R, grad, gpart_gg, gpart_fg, spart);
     return;
   }
   using PS = PassShape<RT>;
@@ -1928,7 +1998,7 @@ __global__ void __launch_bounds__(kT, 2) gd_rows(const float* __restrict__ N, co
   for (int64_t t0 = r0; t0 < r1; t0 += kT) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    tile_load<LD>(N, t0, nt, R, tN);
+    tile_load<LD>(N, t0, nt, ldN, tN);
     tile_load_T<LD>(F, t0, nt, R, tF);
     __syncthreads();
     float af[3] = {0.f, 0.f, 0.f};
@@ -1980,9 +2050,8 @@ __global__ void __launch_bounds__(kT, 2) gd_rows(const float* __restrict__ N, co
     if (threadIdx.x == 0) spart[(size_t)blockIdx.x * 3 + t] = v;
   }
   __syncthreads();
-  double* scratch = reinterpret_cast<double*>(tN);
-  store_gram_partial<RT>(agg, scratch, R, gpart_gg, blockIdx.x);
-  store_gram_partial<RT>(afg, scratch, R, gpart_fg, blockIdx.x);
+  store_gram_partial<RT>(agg, tN, R, gpart_gg, blockIdx.x);
+  store_gram_partial<RT>(afg, tN, R, gpart_fg, blockIdx.x);
 }
 
 // GD update for R <= 32: F <- F - step * grad (step = scal[kStep], 0 after a
@@ -2042,7 +2111,7 @@ __global__ void __launch_bounds__(kT, 2) gd_update_gram(T* __restrict__ F, const
   if constexpr (row_pass_tc<RT>())
     fold_warp_grams<RT>(g, tF, R, gpart, blockIdx.x);
   else
-    store_gram_partial<RT>(a32, reinterpret_cast<double*>(tF), R, gpart, blockIdx.x);
+    store_gram_partial<RT>(a32, tF, R, gpart, blockIdx.x);
 }
 
 // Opt a kernel in to `Bytes` of dynamic shared memory (above the default
@@ -2053,22 +2122,23 @@ cudaError_t opt_in_smem() {
 }
 
 template <int RT>
-__global__ void __launch_bounds__(kT, 2) colnorm_rows(const float* __restrict__ N,
+__global__ void __launch_bounds__(kT, 2) colnorm_rows(const float* __restrict__ N, int ldN,
                                                    const float* __restrict__ W32, int64_t rows, int R,
                                                    double* __restrict__ colsq) {
-  colnorm_rows_body<RT>(N, W32, rows, R, colsq, blockIdx.x, gridDim.x);
+  colnorm_rows_body<RT>(N, ldN, W32, rows, R, colsq, blockIdx.x, gridDim.x);
 }
 
 template <typename T, int RT>
-__global__ void __launch_bounds__(kT, 2) scale_store_rows(const float* __restrict__ N,
+__global__ void __launch_bounds__(kT, 2) scale_store_rows(const float* __restrict__ N, int ldN,
                                                        const float* __restrict__ W32,
                                                        const float* __restrict__ inv,
                                                        const double* __restrict__ lambda,
                                                        int64_t rows, int R, T* __restrict__ F,
+                                                       float* __restrict__ Fpad,
                                                        double* __restrict__ gpart, bool with_ip,
                                                        double* __restrict__ ipart) {
-  scale_store_rows_body<T, RT>(N, W32, inv, lambda, rows, R, F, gpart, with_ip, ipart, blockIdx.x,
-                               gridDim.x);
+  scale_store_rows_body<T, RT>(N, ldN, W32, inv, lambda, rows, R, F, Fpad, gpart, with_ip, ipart,
+                               blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -2108,7 +2178,7 @@ __global__ void __launch_bounds__(kT, 2) colnorm_rows_batch(const DenseJob* __re
                                                          int R) {
   const int j = job_of_block(begin, n, blockIdx.x);
   const DenseJob& J = jobs[j];
-  colnorm_rows_body<RT>(J.N, J.W32, J.rows, R, J.partials, blockIdx.x - begin[j], J.nb);
+  colnorm_rows_body<RT>(J.N, R, J.W32, J.rows, R, J.partials, blockIdx.x - begin[j], J.nb);
 }
 
 template <typename T, int RT>
@@ -2117,8 +2187,8 @@ __global__ void __launch_bounds__(kT, 2) scale_store_rows_batch(const DenseJob* 
                                                              int R, bool last) {
   const int j = job_of_block(begin, n, blockIdx.x);
   const DenseJob& J = jobs[j];
-  scale_store_rows_body<T, RT>(J.N, J.W32, J.inv_lambda, J.lambda, J.rows, R, static_cast<T*>(J.F),
-                               J.partials, last, J.ipart, blockIdx.x - begin[j], J.nb);
+  scale_store_rows_body<T, RT>(J.N, R, J.W32, J.inv_lambda, J.lambda, J.rows, R, static_cast<T*>(J.F),
+                               nullptr, J.partials, last, J.ipart, blockIdx.x - begin[j], J.nb);
 }
 
 __global__ void __launch_bounds__(kT) finish_lambda_batch(const DenseJob* __restrict__ jobs, int R) {
@@ -2238,7 +2308,7 @@ namespace {
 
 // The row passes of one mode for R <= 32 (one thread per row).
 template <typename T, int RT>
-dfacto_status als_post_rows(dfacto_t* h, int mode, float* N) {
+dfacto_status als_post_rows(dfacto_t* h, int mode, const float* N, int ldN) {
   const int R = h->R;
   cudaStream_t s = h->stream;
   const int64_t rows = h->m[mode].dim_o;
@@ -2247,31 +2317,41 @@ dfacto_status als_post_rows(dfacto_t* h, int mode, float* N) {
   constexpr size_t smem = row_pass_smem<RT>();
   DF_CUDA(h, (opt_in_smem<colnorm_rows<RT>, smem>()));
   DF_CUDA(h, (opt_in_smem<scale_store_rows<T, RT>, smem>()));
-  colnorm_rows<RT><<<nb, kT, smem, s>>>(N, h->W32, rows, R, h->partials);
+  float* Fpad = nullptr;  // the padded copy of the new factor comes out of the same pass
+  if (ldN != R) {
+    dfacto_status st;
+    if (!h->pad_F[mode] &&
+        (st = dalloc(h, (void**)&h->pad_F[mode], sizeof(float) * (size_t)rows * ldN)) != DFACTO_OK)
+      return st;
+    Fpad = h->pad_F[mode];
+  }
+  colnorm_rows<RT><<<nb, kT, smem, s>>>(N, ldN, h->W32, rows, R, h->partials);
   DF_COUNT();
   finish_lambda<<<R, kT, 0, s>>>(h->partials, nb, R, h->lambda, h->inv_lambda);
   DF_COUNT();
-  scale_store_rows<T, RT><<<nb, kT, smem, s>>>(N, h->W32, h->inv_lambda, h->lambda, rows, R,
-                                               static_cast<T*>(h->F[mode]), h->partials, last, h->ipart);
+  scale_store_rows<T, RT><<<nb, kT, smem, s>>>(N, ldN, h->W32, h->inv_lambda, h->lambda, rows, R,
+                                               static_cast<T*>(h->F[mode]), Fpad, h->partials, last,
+                                               h->ipart);
   DF_COUNT();
   reduce_partials<<<(R * R + 31) / 32, kT, 0, s>>>(h->partials, nb, R * R, R, false, h->gram[mode]);
   DF_COUNT();
   DF_CUDA(h, cudaGetLastError());
   h->gram_valid[mode] = true;
+  h->pad_valid[mode] = Fpad != nullptr;
   if (last) h->ipart_blocks = nb;
   return DFACTO_OK;
 }
 
 template <typename T>
-dfacto_status als_post_T(dfacto_t* h, int mode, float* N) {
+dfacto_status als_post_T(dfacto_t* h, int mode, const float* N, int ldN) {
   const ModeCSR& M = h->m[mode];
   const int R = h->R;
   const int R4 = (R + 3) / 4;
   cudaStream_t s = h->stream;
-  if (R <= 8) return als_post_rows<T, 8>(h, mode, N);
-  if (R <= 12) return als_post_rows<T, 12>(h, mode, N);
-  if (R <= 16) return als_post_rows<T, 16>(h, mode, N);
-  if (R <= 32) return als_post_rows<T, 32>(h, mode, N);
+  if (R <= 8) return als_post_rows<T, 8>(h, mode, N, ldN);
+  if (R <= 12) return als_post_rows<T, 12>(h, mode, N, ldN);
+  if (R <= 16) return als_post_rows<T, 16>(h, mode, N, ldN);
+  if (R <= 32) return als_post_rows<T, 32>(h, mode, N, ldN);
   const int64_t rows = M.dim_o;
   const unsigned nb = row_blocks(rows);
   const size_t smem_a = solve_bytes(R);
@@ -2316,8 +2396,9 @@ dfacto_status als_pre(dfacto_t* h, int mode) {
 
 // Steps after the MTTKRP N of this mode: N Gamma^{-1}, normalisation, store,
 // and the Gram of the new factor (plus the fit's inner product on mode 3).
-dfacto_status als_post(dfacto_t* h, int mode, float* N) {
-  return h->dtype == DFACTO_BF16 ? als_post_T<__nv_bfloat16>(h, mode, N) : als_post_T<float>(h, mode, N);
+dfacto_status als_post(dfacto_t* h, int mode, const float* N, int ldN) {
+  return h->dtype == DFACTO_BF16 ? als_post_T<__nv_bfloat16>(h, mode, N, ldN)
+                                 : als_post_T<float>(h, mode, N, ldN);
 }
 
 // One mode of Algorithm 2.  Gamma^{-1} depends only on the other two factors,
@@ -2325,6 +2406,8 @@ dfacto_status als_post(dfacto_t* h, int mode, float* N) {
 // passes wait for both.
 dfacto_status als_mode(dfacto_t* h, int mode) {
   dfacto_status st;
+  const float* N = nullptr;
+  int ldN = 0;
   if (h->aux) {
     DF_CUDA(h, cudaEventRecord(h->aux_fork, h->stream));
     DF_CUDA(h, cudaStreamWaitEvent(h->aux, h->aux_fork, 0));
@@ -2333,14 +2416,14 @@ dfacto_status als_mode(dfacto_t* h, int mode) {
     st = als_pre(h, mode);
     h->stream = main;
     cudaError_t e = cudaEventRecord(h->aux_join, h->aux);
-    if (st == DFACTO_OK) st = mttkrp_launch(h, mode, h->N);
+    if (st == DFACTO_OK) st = mttkrp_rows(h, mode, &N, &ldN);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->aux_join, 0);
     if (e != cudaSuccess && st == DFACTO_OK) return cuda_fail(h, e, "auxiliary stream join");
   } else {
     st = als_pre(h, mode);
-    if (st == DFACTO_OK) st = mttkrp_launch(h, mode, h->N);
+    if (st == DFACTO_OK) st = mttkrp_rows(h, mode, &N, &ldN);
   }
-  if (st == DFACTO_OK) st = als_post(h, mode, h->N);
+  if (st == DFACTO_OK) st = als_post(h, mode, N, ldN);
   return st;
 }
 
@@ -2402,7 +2485,9 @@ dfacto_status gd_step_rows(dfacto_t* h) {
     const ModeCSR& M = h->m[mode];
     hadamard_gamma<<<1, 256, 0, s>>>(h->gram[M.f], h->gram[M.in], R, h->lambda_reg, h->W, h->W32);
     DF_COUNT();
-    if ((st = mttkrp_launch(h, mode, h->N)) != DFACTO_OK) return st;
+    const float* N;
+    int ldN;
+    if ((st = mttkrp_rows(h, mode, &N, &ldN)) != DFACTO_OK) return st;
     const int64_t rows = M.dim_o;
     const int nb = pass_blocks(rows);
     const int64_t RR = (int64_t)R * R;
@@ -2411,7 +2496,7 @@ dfacto_status gd_step_rows(dfacto_t* h) {
     double* fg = h->partials + nb * RR;
     double* sp = h->partials + 2 * nb * RR;
     double* P = h->gd_mats + (size_t)mode * 3 * RR;
-    gd_rows<T, RT><<<nb, kT, smem_rows, s>>>(h->N, static_cast<const T*>(h->F[mode]), h->W32, rows, R,
+    gd_rows<T, RT><<<nb, kT, smem_rows, s>>>(N, ldN, static_cast<const T*>(h->F[mode]), h->W32, rows, R,
                                              h->grad[mode], gg, fg, sp);
     DF_COUNT();
     // P0 = F^T F (known), P1 = F^T G + G^T F, P2 = G^T G
@@ -2436,6 +2521,7 @@ dfacto_status gd_step_rows(dfacto_t* h) {
     reduce_partials<<<(R * R + 31) / 32, kT, 0, s>>>(h->partials, nb, R * R, R, false, h->gram[m]);
     DF_COUNT();
     h->gram_valid[m] = true;
+    h->pad_valid[m] = false;
   }
   DF_CUDA(h, cudaGetLastError());
   return DFACTO_OK;
@@ -2488,7 +2574,7 @@ dfacto_status gd_step_T(dfacto_t* h) {
     const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 1023) / 1024, kMaxBlocks * 4));
     gd_update<T><<<nb, 256, 0, s>>>(static_cast<T*>(h->F[m]), h->grad[m], n, h->scal);
     DF_COUNT();
-    h->gram_valid[m] = false;
+    h->gram_valid[m] = h->pad_valid[m] = false;
   }
   DF_CUDA(h, cudaGetLastError());
   for (int m = 0; m < 3; ++m)
@@ -2530,7 +2616,7 @@ dfacto_status apply_step_T(dfacto_t* h) {
     const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 1023) / 1024, kMaxBlocks * 4));
     gd_update<T><<<nb, 256, 0, h->stream>>>(static_cast<T*>(h->F[m]), h->grad[m], n, h->scal);
     DF_COUNT();
-    h->gram_valid[m] = false;
+    h->gram_valid[m] = h->pad_valid[m] = false;
   }
   DF_CUDA(h, cudaGetLastError());
   return DFACTO_OK;

@@ -107,4 +107,9 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// e / d for 0 <= e < 8192 and 1 <= d <= 32 as a multiplication by
+// small_inv(d) = ceil(2^18 / d) and a shift: exact, as e (d - 1) < 2^18.
+__host__ __device__ __forceinline__ uint32_t small_inv(int d) { return ((1u << 18) + (uint32_t)d - 1u) / (uint32_t)d; }
+__device__ __forceinline__ int small_div(int e, uint32_t inv) { return (int)(((uint32_t)e * inv) >> 18); }
+
 }  // namespace dfacto

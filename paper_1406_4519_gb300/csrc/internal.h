@@ -115,14 +115,14 @@ struct dfacto_handle {
   int32_t* carry_row = nullptr;               // [ncta x 4] head row, tail row, slot info
   int64_t carry_cap = 0;                      // CTAs
   int carry_rank = 0;                         // columns of a carry row the buffer holds
-  // MTTKRP at a rank that is not a multiple of four: the two gathered factors
-  // and the output as zero-padded FP32 rows of a multiple of four columns
-  // [max dim x padded rank] each (lazy)
-  float* pad_in = nullptr;
-  float* pad_f = nullptr;
+  // MTTKRP at a rank that is not a multiple of four: the factors as zero-padded
+  // FP32 rows of the walk rank, valid until the factor changes (like gram), and
+  // the output [max dim x walk rank] (all lazy)
+  float* pad_F[3] = {nullptr, nullptr, nullptr};
+  bool pad_valid[3] = {false, false, false};
   float* pad_out = nullptr;
-  // the line search's trilinear pass at such a rank: A, B, C and their
-  // gradients as padded FP32 rows [(dims[0] + dims[1] + dims[2]) x padded rank x 2] (lazy)
+  // the line search's trilinear pass at such a rank: the gradients as padded
+  // FP32 rows [(dims[0] + dims[1] + dims[2]) x walk rank] (lazy)
   float* pad_dual = nullptr;
   double* host_scal = nullptr;                // host mirror of scal
   int32_t* host_flags = nullptr;              // host mirror of flags
@@ -185,6 +185,11 @@ int walk_rank(int R, int vec_opt);
 cudaError_t pad_factor_rows(const void* src, int src_dtype, int64_t rows, int R, int RP, float* dst,
                             cudaStream_t s);
 dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out);
+// The MTTKRP into the handle's own buffer: *N gets its rows of *ld columns (ld is
+// the walk rank; columns past R are zero).
+dfacto_status mttkrp_rows(dfacto_t* h, int mode, const float** N, int* ld);
+// Factor m's padded copy pad_F[m] is up to date afterwards (walk rank != R).
+dfacto_status ensure_padded(dfacto_t* h, int m);
 
 // ---- batches (batch.cu, dense.cu) -----------------------------------------
 // One job of a batch for one mode, as the batched R x R and row kernels see
@@ -232,7 +237,7 @@ void joint_free(dfacto_t* h);
 dfacto_status gram_of_factor(dfacto_t* h, int m);
 dfacto_status als_mode(dfacto_t* h, int mode);
 dfacto_status als_pre(dfacto_t* h, int mode);
-dfacto_status als_post(dfacto_t* h, int mode, float* N);
+dfacto_status als_post(dfacto_t* h, int mode, const float* N, int ldN);
 dfacto_status als_fit(dfacto_t* h);
 dfacto_status fit_direct(dfacto_t* h);
 dfacto_status gd_step(dfacto_t* h);

@@ -610,7 +610,7 @@ dfacto_status joint_rows_side(dfacto_t* h, int side) {
   st = R <= 8 ? joint_solve_side<T, 8>(h, side) : R <= 16 ? joint_solve_side<T, 16>(h, side)
                                                           : joint_solve_side<T, 32>(h, side);
   if (st != DFACTO_OK) return st;
-  h->gram_valid[side] = false;
+  h->gram_valid[side] = h->pad_valid[side] = false;
   return DFACTO_OK;
 }
 

@@ -89,11 +89,25 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
     }
     __syncthreads();
   }
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < dim_o; o += stride) {
-    if (fiber_ptr[o] == fiber_ptr[o + 1]) {
-      float* row = out + o * R;
-      for (int col = 0; col < R; ++col) row[col] = 0.f;
+  // 32 rows per warp: their empty ones as a mask, then the lanes over the rows'
+  // consecutive columns (10M rows of 12 columns, the carries included: 241
+  // us with a thread per row, 120 this way).
+  const int R4 = R / 4;
+  const bool quads = R % 4 == 0;
+  const uint32_t inv = quads ? small_inv(R4) : small_inv(R);
+  const int64_t stride = (int64_t)gridDim.x * kFixThreads;
+  for (int64_t o = ((int64_t)blockIdx.x * kFixThreads + threadIdx.x) & ~(int64_t)31; o < dim_o; o += stride) {
+    const int64_t row = o + lane;
+    const unsigned empty = __ballot_sync(kFull, row < dim_o && fiber_ptr[row] == fiber_ptr[row + 1]);
+    if (empty == 0u) continue;
+    float* dst = out + o * R;
+    if (quads) {
+      for (int e = lane; e < 32 * R4; e += 32)
+        if ((empty >> small_div(e, inv)) & 1u)
+          reinterpret_cast<float4*>(dst)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      for (int e = lane; e < 32 * R; e += 32)
+        if ((empty >> small_div(e, inv)) & 1u) dst[e] = 0.f;
     }
   }
 }
@@ -107,27 +121,42 @@ int next_pow2(int x) {
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 
-// Rows of an R-column matrix (storage type T) as FP32 rows of RP >= R columns,
-// the extra columns zero.
+// Rows of an R-column matrix (storage type T) as FP32 rows of RP >= R columns
+// (RP a multiple of four), the extra columns zero: 32 rows per warp, a lane per
+// four columns of the result.
 template <typename T>
-__global__ void pad_rows(const T* __restrict__ src, int64_t rows, int R, int RP, float* __restrict__ dst) {
-  const int64_t n = rows * RP;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
-    const int64_t r = e / RP;
-    const int c = (int)(e - r * RP);
-    dst[e] = c < R ? to_float(src[r * R + c]) : 0.f;
+__global__ void __launch_bounds__(256) pad_rows(const T* __restrict__ src, int64_t rows, int R, int RP,
+                                                float* __restrict__ dst) {
+  const int lane = threadIdx.x & 31, Q = RP / 4;
+  const uint32_t inv = small_inv(Q);
+  const int64_t stride = (int64_t)gridDim.x * 256;
+  for (int64_t r0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) & ~(int64_t)31; r0 < rows; r0 += stride) {
+    const int n = (int)min((int64_t)32, rows - r0) * Q;
+    for (int e = lane; e < n; e += 32) {
+      const int r = small_div(e, inv), c = 4 * (e - r * Q);
+      const T* q = src + (r0 + r) * R + c;
+      float4 v;
+      v.x = to_float(q[0]);  // c < R: fewer than four columns are added
+      v.y = c + 1 < R ? to_float(q[1]) : 0.f;
+      v.z = c + 2 < R ? to_float(q[2]) : 0.f;
+      v.w = c + 3 < R ? to_float(q[3]) : 0.f;
+      reinterpret_cast<float4*>(dst + r0 * RP)[e] = v;
+    }
   }
 }
 
 // The first R of every RP columns back to rows of R columns.
-__global__ void unpad_rows(const float* __restrict__ src, int64_t rows, int R, int RP, float* __restrict__ dst) {
-  const int64_t n = rows * R;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
-    const int64_t r = e / R;
-    const int c = (int)(e - r * R);
-    dst[e] = src[r * RP + c];
+__global__ void __launch_bounds__(256) unpad_rows(const float* __restrict__ src, int64_t rows, int R, int RP,
+                                                  float* __restrict__ dst) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t inv = small_inv(R);
+  const int64_t stride = (int64_t)gridDim.x * 256;
+  for (int64_t r0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) & ~(int64_t)31; r0 < rows; r0 += stride) {
+    const int n = (int)min((int64_t)32, rows - r0) * R;
+    for (int e = lane; e < n; e += 32) {
+      const int r = small_div(e, inv);
+      dst[r0 * R + e] = src[(r0 + r) * RP + (e - r * R)];
+    }
   }
 }
 
@@ -145,10 +174,10 @@ cudaError_t pad_factor_rows(const void* src, int src_dtype, int64_t rows, int R,
                             cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
   if (src_dtype == DFACTO_BF16)
-    pad_rows<__nv_bfloat16><<<rows_grid(rows * RP), 256, 0, s>>>(static_cast<const __nv_bfloat16*>(src),
+    pad_rows<__nv_bfloat16><<<rows_grid(rows), 256, 0, s>>>(static_cast<const __nv_bfloat16*>(src),
                                                                    rows, R, RP, dst);
   else
-    pad_rows<float><<<rows_grid(rows * RP), 256, 0, s>>>(static_cast<const float*>(src), rows, R, RP, dst);
+    pad_rows<float><<<rows_grid(rows), 256, 0, s>>>(static_cast<const float*>(src), rows, R, RP, dst);
   DF_COUNT();
   return cudaGetLastError();
 }
@@ -205,17 +234,32 @@ WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, in
   return c;
 }
 
-dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out) {
+// The padded FP32 copy of factor m (rank RP), made when the factor changed.
+dfacto_status ensure_padded(dfacto_t* h, int m) {
+  const int RP = walk_rank(h->R, h->opt.vec);
+  if (h->pad_valid[m]) return DFACTO_OK;
+  dfacto_status st;
+  if (!h->pad_F[m] &&
+      (st = dalloc(h, reinterpret_cast<void**>(&h->pad_F[m]), sizeof(float) * (size_t)h->dims[m] * RP)) != DFACTO_OK)
+    return st;
+  DF_CUDA(h, pad_factor_rows(h->F[m], h->dtype, h->dims[m], h->R, RP, h->pad_F[m], h->stream));
+  h->pad_valid[m] = true;
+  return DFACTO_OK;
+}
+
+namespace {
+
+// The walk and its fix-up.  At a rank that is not a multiple of four the walk
+// runs on zero-padded FP32 copies of the two gathered factors at the padded
+// rank RP (one 16-byte gather per lane: R = 10 walks 3 of 4 lanes per group
+// instead of 5 of 8 with 8-byte gathers, measured 1.45x faster); an explicit
+// lane width keeps the unpadded walk.  Both walks pad alike, so they still
+// compute the same sums in the same order.  The result (rows of RP columns) goes
+// to `wout`.
+dfacto_status walk_rows(dfacto_t* h, int mode, float* wout) {
   ModeCSR& M = h->m[mode];
-  // At a rank that is not a multiple of four the walk runs on zero-padded FP32
-  // copies of the two gathered factors at the padded rank RP (one 16-byte
-  // gather per lane: R = 10 walks 3 of 4 lanes per group instead of 5 of 8
-  // with 8-byte gathers, measured 1.45x faster) and its output is copied back
-  // to R columns; an explicit lane width keeps the unpadded walk.  Both walks
-  // pad alike, so they still compute the same sums in the same order.
-  const int R = h->R;
-  const int RP = walk_rank(R, h->opt.vec);
-  const bool padded = RP != R;
+  const int RP = walk_rank(h->R, h->opt.vec);
+  const bool padded = RP != h->R;
   const WalkCfg cfg = M.cfg;
   dfacto_status st = ensure_segments(h, mode);
   if (st != DFACTO_OK) return st;
@@ -240,17 +284,11 @@ dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out) {
   }
   const void* Fin = h->F[M.in];
   const void* Ff = h->F[M.f];
-  float* wout = out;
   if (padded) {
-    const int64_t maxdim = std::max<int64_t>(h->dims[0], std::max<int64_t>(h->dims[1], h->dims[2]));
-    const size_t bytes = sizeof(float) * (size_t)maxdim * RP;
-    for (float** q : {&h->pad_in, &h->pad_f, &h->pad_out})
-      if (!*q && (st = dalloc(h, reinterpret_cast<void**>(q), bytes)) != DFACTO_OK) return st;
-    DF_CUDA(h, pad_factor_rows(Fin, h->dtype, h->dims[M.in], R, RP, h->pad_in, h->stream));
-    DF_CUDA(h, pad_factor_rows(Ff, h->dtype, h->dims[M.f], R, RP, h->pad_f, h->stream));
-    Fin = h->pad_in;
-    Ff = h->pad_f;
-    wout = h->pad_out;
+    if ((st = ensure_padded(h, M.in)) != DFACTO_OK) return st;
+    if ((st = ensure_padded(h, M.f)) != DFACTO_OK) return st;
+    Fin = h->pad_F[M.in];
+    Ff = h->pad_F[M.f];
   }
   MttkrpParams a;
   a.fiber_ptr = M.fiber_ptr;
@@ -286,12 +324,39 @@ dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out) {
   }
   DF_CUDA(h, launch_mttkrp_fixup(h->carry_row, h->carry, M.fiber_ptr, M.nz_ptr, wout, RP, P, ncta,
                                  M.dim_o, h->flags + kFlagInternal, h->stream));
-  if (padded) {
-    unpad_rows<<<rows_grid(M.dim_o * R), 256, 0, h->stream>>>(h->pad_out, M.dim_o, R, RP, out);
-    DF_COUNT();
-    DF_CUDA(h, cudaGetLastError());
-  }
   return DFACTO_OK;
+}
+
+dfacto_status ensure_pad_out(dfacto_t* h, int RP) {
+  if (h->pad_out) return DFACTO_OK;
+  const int64_t maxdim = std::max<int64_t>(h->dims[0], std::max<int64_t>(h->dims[1], h->dims[2]));
+  return dalloc(h, reinterpret_cast<void**>(&h->pad_out), sizeof(float) * (size_t)maxdim * RP);
+}
+
+}  // namespace
+
+dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out) {
+  const int R = h->R, RP = walk_rank(R, h->opt.vec);
+  if (RP == R) return walk_rows(h, mode, out);
+  dfacto_status st = ensure_pad_out(h, RP);
+  if (st == DFACTO_OK) st = walk_rows(h, mode, h->pad_out);
+  if (st != DFACTO_OK) return st;
+  const int64_t rows = h->m[mode].dim_o;
+  unpad_rows<<<rows_grid(rows), 256, 0, h->stream>>>(h->pad_out, rows, R, RP, out);
+  DF_COUNT();
+  DF_CUDA(h, cudaGetLastError());
+  return DFACTO_OK;
+}
+
+dfacto_status mttkrp_rows(dfacto_t* h, int mode, const float** N, int* ld) {
+  const int RP = walk_rank(h->R, h->opt.vec);
+  *ld = RP;
+  *N = h->N;
+  if (RP == h->R) return walk_rows(h, mode, h->N);
+  const dfacto_status st = ensure_pad_out(h, RP);
+  if (st != DFACTO_OK) return st;
+  *N = h->pad_out;
+  return walk_rows(h, mode, h->pad_out);
 }
 
 }  // namespace dfacto
