@@ -33,6 +33,7 @@ struct DualParams {
   const float* nz_val;
   const int32_t* seg_fib;
   const uint32_t* end_bits;  // dual_walk2: bit p set iff nonzero p ends its fiber
+  const uint32_t* row_bits;  // dual_walk2: bit p set iff nonzero p starts its row
   const void* A;
   const void* B;
   const void* C;
@@ -165,217 +166,194 @@ __global__ void __launch_bounds__(kWalkWarps * 32) dual_walk(const DualParams a)
 }
 
 // ---------------------------------------------------------------------------
-// dual_walk2: the same four terms with the organisation of mttkrp_walk2: fiber
-// ends from the end bitmask of the mode-1 copy, both fiber sums (vB, vG) parked
-// in shared memory where a fiber ends, and the closed fibers folded CC at a
-// time (their C and GC rows gathered together).  At most 8 values of each of
-// the two gathered rows (B and GB) are in flight per lane.
+// dual_walk2: the same four terms with the organisation of mttkrp_walk2: per
+// batch of B positions a group's lanes hold their positions' (j, x) and the k of
+// their fibers, and per sub-batch of U positions gather the B and GB rows and the
+// C and GC rows of the fibers that end there together.  Each lane keeps two
+// fiber sums and three row sums.
+//
+// Bound by the latency of its gathers against the registers that hold them, like
+// mttkrp_walk2.  50M power-law nonzeros, R = 32: 2.30 ms with the fiber sums
+// parked in shared memory and folded after a second round of loads, 1.97 now;
+// R = 10 (padded to 12): a GD step 4.59 -> 3.29 ms with the walks and row passes.
 // ---------------------------------------------------------------------------
-// A thread's VEC parked floats in shared memory.  Slot k of thread tid holds
-// them as VEC/4 float4 chunks, chunk q at ((k * VEC/4 + q) * NT + tid) * 4, so
-// that a warp's accesses to one chunk are consecutive 16-byte words (no bank
-// conflicts); VEC < 4 keeps the VEC floats together at (k * NT + tid) * VEC.
-template <int VEC, int NT>
-__device__ __forceinline__ float* park_slot(float* vb, int k, int tid) {
-  if constexpr (VEC % 4 == 0) return vb + ((size_t)k * (VEC / 4) * NT + tid) * 4;
-  else return vb + ((size_t)k * NT + tid) * VEC;
-}
-template <int VEC, int NT>
-__device__ __forceinline__ void smem_st(float* p, const float (&v)[VEC]) {
-  if constexpr (VEC % 4 == 0) {
-#pragma unroll
-    for (int e = 0; e < VEC; e += 4)
-      *reinterpret_cast<float4*>(p + (size_t)(e / 4) * NT * 4) =
-          make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-  } else if constexpr (VEC == 2) {
-    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-  } else {
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) p[e] = v[e];
-  }
-}
-template <int VEC, int NT>
-__device__ __forceinline__ void smem_ld(const float* p, float (&v)[VEC]) {
-  if constexpr (VEC % 4 == 0) {
-#pragma unroll
-    for (int e = 0; e < VEC; e += 4) {
-      const float4 t = *reinterpret_cast<const float4*>(p + (size_t)(e / 4) * NT * 4);
-      v[e] = t.x; v[e + 1] = t.y; v[e + 2] = t.z; v[e + 3] = t.w;
-    }
-  } else if constexpr (VEC == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(p);
-    v[0] = t.x; v[1] = t.y;
-  } else {
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) v[e] = p[e];
-  }
-}
+// Positions gathered together, at most (two: 128 registers, two CTAs per SM,
+// without spills; four spill and take 5% longer, two at 80 registers 20%).
+constexpr int kDualGathers = 2;
 
+// If `on` is nonzero: u1 += c vG, u2 += (sC g) vB, u3 += (sC g) vG, vB = vG = 0.
 template <int VEC>
-struct Dual2Shape {
-  static constexpr int NT = kWalkWarps * 32;
-  static constexpr int U = 8 / VEC > 0 ? 8 / VEC : 1;  // capped by G below
-  static constexpr int CC = 2;                           // fibers folded per round
-};
+__device__ __forceinline__ void fold_dual_if(uint32_t on, const Cols<VEC>& cf, const Cols<VEC>& gcf, float sC,
+                                             Cols<VEC>& vB, Cols<VEC>& vG, Cols<VEC>& u1, Cols<VEC>& u2,
+                                             Cols<VEC>& u3) {
+  if (!on) return;
+  float c[VEC], g[VEC], b[VEC], w[VEC], a1[VEC], a2[VEC], a3[VEC];
+  cf.unpack(c);
+  gcf.unpack(g);
+  vB.unpack(b);
+  vG.unpack(w);
+  u1.unpack(a1);
+  u2.unpack(a2);
+  u3.unpack(a3);
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) {
+    const float gs = g[e] * sC;
+    a1[e] = fmaf(c[e], w[e], a1[e]);
+    a2[e] = fmaf(gs, b[e], a2[e]);
+    a3[e] = fmaf(gs, w[e], a3[e]);
+  }
+  u1.pack(a1);
+  u2.pack(a2);
+  u3.pack(a3);
+  vB.zero();
+  vG.zero();
+}
 
 template <typename T, int VEC, int G>
-__global__ void __launch_bounds__(kWalkWarps * 32, 3) dual_walk2(const DualParams a) {
-  constexpr int NG = 32 / G;
-  constexpr int SEGS = kWalkWarps * NG;
-  constexpr int NT = Dual2Shape<VEC>::NT;
-  constexpr int U = G < Dual2Shape<VEC>::U ? G : Dual2Shape<VEC>::U;
-  constexpr int CC = Dual2Shape<VEC>::CC < U ? Dual2Shape<VEC>::CC : U;
-  extern __shared__ __align__(16) float vb[];  // 2U slots of NT x VEC parked sums
+__global__ void __launch_bounds__(kWalkWarps * 32, 2) dual_walk2(const DualParams a) {
+  constexpr int NG = 32 / G, SEGS = kWalkWarps * NG, LPP = G >= 8 ? 1 : 2, B = G * LPP;
+  constexpr int U = kDualGathers < B ? kDualGathers : B;
+  constexpr uint32_t kBatch = B == 32 ? 0xffffffffu : (1u << (B & 31)) - 1u;
+  static_assert(B % U == 0 && U % LPP == 0, "batch layout");
   __shared__ double s_t[kWalkWarps][4];
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int g = lane / G, c = lane % G;
-  const int gbase = g * G;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane / G, c = lane % G, gbase = g * G;
   const int col0 = c * VEC;
   const bool colok = col0 < a.R;
-  const int sl = warp * NG + g;
-  const int nnz = (int)a.nnz;
-  const int p0 = (int)min(((int64_t)blockIdx.x * SEGS + sl) * a.seg, a.nnz);
+  const int R = a.R;
+  const int nnz = (int)a.nnz, npad = (int)walk_padded(a.nnz);
+  const int64_t sl = (int64_t)blockIdx.x * SEGS + warp * NG + g;
+  const int p0 = (int)min(sl * a.seg, (int64_t)npad);
   const int p1 = min(p0 + a.seg, nnz);
   const bool active = p0 < nnz;
-  const int R = a.R;
-  const T* __restrict__ A = static_cast<const T*>(a.A);
-  const T* __restrict__ B = static_cast<const T*>(a.B);
-  const T* __restrict__ C = static_cast<const T*>(a.C);
+  const int cl = colok ? col0 : 0;  // lanes past column R walk column 0 and add nothing
   const float sA = a.gscale[0], sB = a.gscale[1], sC = a.gscale[2];
+  auto rowT = [&](const void* F, int t) { return static_cast<const T*>(F) + ((uint64_t)(uint32_t)t * (uint32_t)R + cl); };
+  auto rowG = [&](const float* F, int t) { return F + ((uint64_t)(uint32_t)t * (uint32_t)R + cl); };
 
-  float vB[VEC], vG[VEC], u1[VEC], u2[VEC], u3[VEC];
-#pragma unroll
-  for (int e = 0; e < VEC; ++e) vB[e] = vG[e] = u1[e] = u2[e] = u3[e] = 0.f;
+  Cols<VEC> vB, vG, u1, u2, u3;
+  vB.zero(); vG.zero(); u1.zero(); u2.zero(); u3.zero();
   float t[4] = {0.f, 0.f, 0.f, 0.f};
-  int q = 0, row_cur = -1;
+  int q = 0, row_cur = 0;
+  uint32_t ew = 0u, rw = 0u;
   if (active) {
-    q = a.seg_fib[(int64_t)blockIdx.x * SEGS + sl];
+    q = a.seg_fib[sl];
     row_cur = a.fiber_row[q];
+    ew = __ldg(a.end_bits + (p0 >> 5));
+    rw = __ldg(a.row_bits + (p0 >> 5)) & ~1u;
   }
   // Close row row_cur: T110 += GA.u1, T101 += GA.u2, T011 += A.u3, T111 += GA.u3.
   auto emit_row = [&]() {
     if (colok) {
-      float ar[VEC], gar[VEC];
-      VecIO<T, VEC>::load(A + (int64_t)row_cur * R + col0, ar);
-      VecIO<float, VEC>::load(a.GA + (int64_t)row_cur * R + col0, gar);
+      float ar[VEC], gar[VEC], x1[VEC], x2[VEC], x3[VEC];
+      VecIO<T, VEC>::load(rowT(a.A, row_cur), ar);
+      VecIO<float, VEC>::load(rowG(a.GA, row_cur), gar);
+      u1.unpack(x1);
+      u2.unpack(x2);
+      u3.unpack(x3);
 #pragma unroll
       for (int e = 0; e < VEC; ++e) {
         const float ga = gar[e] * sA;
-        t[0] = fmaf(ga, u1[e], t[0]);
-        t[1] = fmaf(ga, u2[e], t[1]);
-        t[2] = fmaf(ar[e], u3[e], t[2]);
-        t[3] = fmaf(ga, u3[e], t[3]);
+        t[0] = fmaf(ga, x1[e], t[0]);
+        t[1] = fmaf(ga, x2[e], t[1]);
+        t[2] = fmaf(ar[e], x3[e], t[2]);
+        t[3] = fmaf(ga, x3[e], t[3]);
       }
     }
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) u1[e] = u2[e] = u3[e] = 0.f;
+    u1.zero();
+    u2.zero();
+    u3.zero();
   };
-  // Fold a closed fiber (row r, sums pB / pG, rows cf = C[k], gcf = GC[k]).
-  auto fold = [&](int r, const float (&pB)[VEC], const float (&pG)[VEC], const float (&cf)[VEC],
-                  const float (&gcf)[VEC]) {
-    if (r != row_cur) {
-      emit_row();
-      row_cur = r;
-    }
+  auto load_stream = [&](int p, int (&in)[LPP], int (&x)[LPP]) {
+    const int pl = min(p, npad - B) + c * LPP;
+    ldg_words<LPP>(a.nz_idx + pl, in);
+    ldg_words<LPP>(reinterpret_cast<const int32_t*>(a.nz_val) + pl, x);
+  };
+  auto load_fibers = [&](int qb, uint32_t e, int (&f)[LPP]) {
 #pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-      u1[e] = fmaf(cf[e], pG[e], u1[e]);
-      u2[e] = fmaf(gcf[e], pB[e], u2[e]);
-      u3[e] = fmaf(gcf[e], pG[e], u3[e]);
-    }
+    for (int j = 0; j < LPP; ++j)
+      f[j] = __ldg(a.fiber_idx + (qb + __popc(e & ((1u << (c * LPP + j)) - 1u))));
   };
 
-  for (int base = p0; base < p0 + a.seg; base += G) {
-    const int pl = base + c;
-    const bool okl = pl < p1;
-    const int my_in = okl ? __ldg(a.nz_idx + pl) : 0;
-    const float my_x = okl ? __ldg(a.nz_val + pl) : 0.f;
-    const uint32_t ebits =
-        (active && base < p1) ? (__ldg(a.end_bits + (base >> 5)) >> (base & 31)) : 0u;
-#pragma unroll
-    for (int u0 = 0; u0 < G; u0 += U) {
-      float b[U][VEC], gb[U][VEC];
-#pragma unroll
-      for (int uu = 0; uu < U; ++uu) {
-        const int j = __shfl_sync(kFull, my_in, gbase + u0 + uu);
-        if (colok && base + u0 + uu < p1) {
-          VecIO<T, VEC>::load(B + (int64_t)j * R + col0, b[uu]);
-          VecIO<float, VEC>::load(a.GB + (int64_t)j * R + col0, gb[uu]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) b[uu][e] = gb[uu][e] = 0.f;
-        }
+  int in[LPP], x[LPP], f[LPP];
+  load_stream(p0, in, x);
+  load_fibers(q, ew, f);
+  for (int pb = p0; pb < p0 + a.seg; pb += 32) {
+    uint32_t ewn = 0u, rwn = 0u;  // the next 32 positions' bits
+    if (pb + 32 < p1) {
+      ewn = __ldg(a.end_bits + ((pb + 32) >> 5));
+      rwn = __ldg(a.row_bits + ((pb + 32) >> 5));
+    }
+#pragma unroll 1
+    for (int k = 0; k < 32 / B; ++k) {
+      const uint32_t eb = ew & kBatch, rb = rw & kBatch;
+      const int qn = q + __popc(eb);
+      if constexpr (B < 32) {
+        ew = k == 32 / B - 1 ? ewn : ew >> (B & 31);
+        rw = k == 32 / B - 1 ? rwn : rw >> (B & 31);
+      } else {
+        ew = ewn;
+        rw = rwn;
       }
-      int k = 0;
+      int in_n[LPP], x_n[LPP], f_n[LPP];
+      load_stream(pb + (k + 1) * B, in_n, x_n);
+      load_fibers(qn, ew, f_n);
+      auto batch = [&](auto with_rows) {
+#pragma unroll 1
+        for (int u0 = 0; u0 < B; u0 += U) {
+          RawCols<T, VEC> bi[U], ci[U];
+          RawCols<float, VEC> gb[U], gc[U];
+          const int src = gbase + u0 / LPP;
+          const uint32_t e4 = eb >> u0;
 #pragma unroll
-      for (int uu = 0; uu < U; ++uu) {
-        const float x = __shfl_sync(kFull, my_x, gbase + u0 + uu);
-        const int p = base + u0 + uu;
+          for (int uu = 0; uu < U; ++uu) {
+            const int j = G == 1 ? in[uu % LPP] : __shfl_sync(kFull, in[uu % LPP], src + uu / LPP);
+            bi[uu].load(rowT(a.B, j));
+            gb[uu].load(rowG(a.GB, j));
+          }
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) {
-          vB[e] = fmaf(x, b[uu][e], vB[e]);
-          vG[e] = fmaf(x, gb[uu][e] * sB, vG[e]);
-        }
-        const bool end = p < p1 && ((ebits >> (u0 + uu)) & 1u);
-        if (end) {
-          smem_st<VEC, NT>(park_slot<VEC, NT>(vb, 2 * k, tid), vB);
-          smem_st<VEC, NT>(park_slot<VEC, NT>(vb, 2 * k + 1, tid), vG);
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) vB[e] = vG[e] = 0.f;
-        }
-        k += end ? 1 : 0;
-      }
-      for (int j0 = 0; j0 < k; j0 += CC) {
-        int rj[CC];
-        float cf[CC][VEC], gcf[CC][VEC];
-#pragma unroll
-        for (int j = 0; j < CC; ++j) {
-          rj[j] = row_cur;
-          if (j0 + j < k) {
-            const int kk = __ldg(a.fiber_idx + q + j0 + j);
-            rj[j] = __ldg(a.fiber_row + q + j0 + j);
-            if (colok) {
-              VecIO<T, VEC>::load(C + (int64_t)kk * R + col0, cf[j]);
-              VecIO<float, VEC>::load(a.GC + (int64_t)kk * R + col0, gcf[j]);
+          for (int uu = 0; uu < U; ++uu) {
+            const int kk = G == 1 ? f[uu % LPP] : __shfl_sync(kFull, f[uu % LPP], src + uu / LPP);
+            if (e4 & (1u << uu)) {
+              ci[uu].load(rowT(a.C, kk));
+              gc[uu].load(rowG(a.GC, kk));
             }
           }
-          if (!(j0 + j < k && colok)) {
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) cf[j][e] = gcf[j][e] = 0.f;
+          for (int uu = 0; uu < U; ++uu) {
+            const float xu = __int_as_float(G == 1 ? x[uu % LPP] : __shfl_sync(kFull, x[uu % LPP], src + uu / LPP));
+            if constexpr (decltype(with_rows)::value) {
+              if ((rb >> (u0 + uu)) & 1u) {
+                emit_row();
+                row_cur = __ldg(a.fiber_row + (q + __popc(eb & ((1u << (u0 + uu)) - 1u))));
+              }
+            }
+            axpy_cols<VEC>(xu, bi[uu].get(), vB);
+            axpy_cols<VEC>(xu * sB, gb[uu].get(), vG);  // a power of two scales exactly
+            fold_dual_if<VEC>(e4 & (1u << uu), ci[uu].get(), gc[uu].get(), sC, vB, vG, u1, u2, u3);
           }
         }
+      };
+      if (__any_sync(kFull, rb != 0u)) batch(std::true_type{});
+      else batch(std::false_type{});
+      q = qn;
 #pragma unroll
-        for (int j = 0; j < CC; ++j) {
-          if (j0 + j < k) {
-            float pB[VEC], pG[VEC];
-            smem_ld<VEC, NT>(park_slot<VEC, NT>(vb, 2 * (j0 + j), tid), pB);
-            smem_ld<VEC, NT>(park_slot<VEC, NT>(vb, 2 * (j0 + j) + 1, tid), pG);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) gcf[j][e] *= sC;
-            fold(rj[j], pB, pG, cf[j], gcf[j]);
-          }
-        }
+      for (int j = 0; j < LPP; ++j) {
+        in[j] = in_n[j];
+        x[j] = x_n[j];
+        f[j] = f_n[j];
       }
-      q += k;
     }
   }
   if (active) {
     // the fiber open at the segment end (its last nonzero lies beyond p1)
     if (!((__ldg(a.end_bits + ((p1 - 1) >> 5)) >> ((p1 - 1) & 31)) & 1u)) {
+      RawCols<T, VEC> cr;
+      RawCols<float, VEC> gr;
       const int kk = __ldg(a.fiber_idx + q);
-      const int r = __ldg(a.fiber_row + q);
-      float cf[VEC], gcf[VEC];
-      if (colok) {
-        VecIO<T, VEC>::load(C + (int64_t)kk * R + col0, cf);
-        VecIO<float, VEC>::load(a.GC + (int64_t)kk * R + col0, gcf);
-      } else {
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) cf[e] = gcf[e] = 0.f;
-      }
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) gcf[e] *= sC;
-      fold(r, vB, vG, cf, gcf);
+      cr.load(rowT(a.C, kk));
+      gr.load(rowG(a.GC, kk));
+      fold_dual_if<VEC>(1u, cr.get(), gr.get(), sC, vB, vG, u1, u2, u3);
     }
     emit_row();
   }
@@ -391,12 +369,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 3) dual_walk2(const DualParam
     for (int w = 0; w < kWalkWarps; ++w) sum += s_t[w][threadIdx.x];
     a.part[(size_t)blockIdx.x * 4 + threadIdx.x] = sum;
   }
-}
-
-template <int VEC, int G>
-size_t dual2_smem() {
-  constexpr int U = G < Dual2Shape<VEC>::U ? G : Dual2Shape<VEC>::U;
-  return sizeof(float) * (size_t)2 * U * Dual2Shape<VEC>::NT * VEC;
 }
 
 // scal[kT110 + k] = sum over CTAs of part[b][k], k = 0..3 (fixed order:
@@ -451,11 +423,14 @@ __global__ void grad_scales(const unsigned* __restrict__ maxbits, float* __restr
 
 template <typename T, int VEC, int G>
 cudaError_t go(const DualParams& a, int64_t ncta, cudaStream_t s, int kernel) {
-  if (kernel == 2) {
-    dual_walk2<T, VEC, G><<<(unsigned)ncta, kWalkWarps * 32, dual2_smem<VEC, G>(), s>>>(a);
-  } else {
-    dual_walk<T, VEC, G><<<(unsigned)ncta, kWalkWarps * 32, 0, s>>>(a);
+  if constexpr (VEC <= 4) {
+    if (kernel == 2) {
+      dual_walk2<T, VEC, G><<<(unsigned)ncta, kWalkWarps * 32, 0, s>>>(a);
+      DF_COUNT();
+      return cudaGetLastError();
+    }
   }
+  dual_walk<T, VEC, G><<<(unsigned)ncta, kWalkWarps * 32, 0, s>>>(a);
   DF_COUNT();
   return cudaGetLastError();
 }
@@ -478,8 +453,8 @@ dfacto_status dual_pass(dfacto_t* h) {
   ModeCSR& M = h->m[0];
   dfacto_status st = ensure_segments(h, 0);
   if (st != DFACTO_OK) return st;
-  // The mode-1 walk's segments; dual_walk2 keeps five accumulators and two
-  // gathered rows per lane, so its lanes take at most four columns.  At a rank
+  // The mode-1 walk's segments; dual_walk2 keeps five sums and two gathered rows
+  // per position and lane, so its lanes take at most four columns.  At a rank
   // that is not a multiple of four it walks zero-padded FP32 copies of the
   // factors and gradients at the rank rounded up, as the MTTKRP does (the zero
   // columns add nothing to the four terms).
@@ -516,17 +491,15 @@ dfacto_status dual_pass(dfacto_t* h) {
   if (padded) {
     const int64_t rows = (int64_t)h->dims[0] + h->dims[1] + h->dims[2];
     if (!h->pad_dual &&
-        (st = dalloc(h, (void**)&h->pad_dual, sizeof(float) * 2 * (size_t)rows * RP)) != DFACTO_OK)
+        (st = dalloc(h, (void**)&h->pad_dual, sizeof(float) * (size_t)rows * RP)) != DFACTO_OK)
       return st;
     float* q = h->pad_dual;
     for (int m = 0; m < 3; ++m) {
-      float* pf = q;
-      float* pg = q + (size_t)h->dims[m] * RP;
-      DF_CUDA(h, pad_factor_rows(h->F[m], h->dtype, h->dims[m], R, RP, pf, h->stream));
-      DF_CUDA(h, pad_factor_rows(h->grad[m], DFACTO_F32, h->dims[m], R, RP, pg, h->stream));
-      Fm[m] = pf;
-      Gm[m] = pg;
-      q += 2 * (size_t)h->dims[m] * RP;
+      if ((st = ensure_padded(h, m)) != DFACTO_OK) return st;
+      DF_CUDA(h, pad_factor_rows(h->grad[m], DFACTO_F32, h->dims[m], R, RP, q, h->stream));
+      Fm[m] = h->pad_F[m];
+      Gm[m] = q;
+      q += (size_t)h->dims[m] * RP;
     }
   }
   DualParams a;
@@ -537,6 +510,7 @@ dfacto_status dual_pass(dfacto_t* h) {
   a.nz_val = M.nz_val;
   a.seg_fib = M.seg_fib;
   a.end_bits = M.end_bits;
+  a.row_bits = M.row_bits;
   a.A = Fm[0];
   a.B = Fm[1];
   a.C = Fm[2];

@@ -428,12 +428,17 @@ struct Cols {
 #pragma unroll
     for (int e = 0; e < VEC / 2; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(o[2 * e]), "=f"(o[2 * e + 1]) : "l"(p[e]));
   }
+  __device__ __forceinline__ void pack(const float (&v)[VEC]) {
+#pragma unroll
+    for (int e = 0; e < VEC / 2; ++e) asm("mov.b64 %0, {%1, %2};" : "=l"(p[e]) : "f"(v[2 * e]), "f"(v[2 * e + 1]));
+  }
 };
 template <>
 struct Cols<1> {
   float p[1];
   __device__ __forceinline__ void zero() { p[0] = 0.f; }
   __device__ __forceinline__ void unpack(float (&o)[1]) const { o[0] = p[0]; }
+  __device__ __forceinline__ void pack(const float (&v)[1]) { p[0] = v[0]; }
 };
 
 // v += x w.
