@@ -142,9 +142,10 @@ __device__ __forceinline__ float ld_f(const __nv_bfloat16* p) { return __bfloat1
 // end (slot 1); the row's block adds its pieces in order.
 //
 // 100,000 users x 50,000 items x 20,000 words, 2M ratings, R = 16: 63.4 ms per
-// sweep with a warp per row (most of it one user's ratings), 3.0 ms now.
+// sweep with a warp per row (most of it one user's ratings), 2.2 ms now (3.0 with
+// pieces of 1,024: the rows just below that length share a few blocks).
 // ---------------------------------------------------------------------------
-constexpr int kHeavyRatings = 1024;
+constexpr int kHeavyRatings = 256;
 constexpr int kJTileLd = 33;  // rows of a block, padded
 
 // RP: R padded to 8, 16 or 32 columns.  Lane (i, h), i = lane % RP, h = lane /
@@ -212,11 +213,13 @@ __device__ __forceinline__ void joint_accumulate(const int32_t* __restrict__ yco
 #pragma unroll
       for (int c = 0; c < S::CPL; ++c) hrow[c] = fmaf(vi, w[c], hrow[c]);
     }
-    // the groups take every CG-th rating of the right side
+    // the groups take every CG-th rating of the right side (conversions run on
+    // the FP64 pipe too: y is converted once, a rating per lane)
+    const double yd = y;
     for (int t0 = 0; t0 < n; t0 += S::CG) {
       const int t = t0 + h;  // < 32
-      const float yt = __shfl_sync(kFull, y, t);
-      if (t < n) rhs += (double)yt * (double)tile[t * S::LD + i];
+      const double yt = __shfl_sync(kFull, yd, t);
+      if (t < n) rhs += yt * (double)tile[t * S::LD + i];
     }
   }
 #pragma unroll
@@ -289,32 +292,17 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
   float* tiles = reinterpret_cast<float*>(jsm + (((size_t)(jtri(R) + R) * kJTileLd + 1) & ~(size_t)1));
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane % RP, h = lane / RP;
   const int64_t ntiles = (rows + 31) / 32;
+  // blocks that share an SM solve on different warp schedulers (each retires
+  // half an FP64 lane per clock)
+  const int solver = (blockIdx.x / 152) % kJSolveWarps;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int nr = (int)min((int64_t)32, rows - 32 * tile);
+    // rows tile, tile + ntiles, ...: neighbouring rows, which rate alike where
+    // labels are ordered by use, go to different blocks
+    const int nr = (int)((rows - tile + ntiles - 1) / ntiles);  // <= 32
     for (int rr = warp; rr < nr; rr += kJSolveWarps) {
-      const int64_t row = 32 * tile + rr;
+      const int64_t row = tile + rr * ntiles;
       const int64_t b = yptr ? yptr[row] : 0, e = yptr ? yptr[row + 1] : 0;
-      if (e - b > kHeavyRatings) {
-        // the row's pieces in order, a lane per entry
-        const int64_t k0 = b / kHeavyRatings, k1 = (e - 1) / kHeavyRatings;
-        const int s0 = b % kHeavyRatings ? 1 : 0;
-        for (int t = lane; t < jtri(R); t += 32) {
-          int ti = 0;
-          while (jtri(ti + 1) <= t) ++ti;
-          double a = 0.0;
-          for (int64_t k = k0; k <= k1; ++k)
-            a += (double)reinterpret_cast<const float*>(slots + (2 * k + (k == k0 ? s0 : 0)) * jslot_bytes(R))[t];
-          Hs[t * kJTileLd + rr] = base[ti * R + (t - jtri(ti))] + a;
-        }
-        for (int t = lane; t < R; t += 32) {
-          double a = mu * (double)N[row * R + t];
-          for (int64_t k = k0; k <= k1; ++k)
-            a += reinterpret_cast<const double*>(slots + (2 * k + (k == k0 ? s0 : 0) + 1) * jslot_bytes(R) -
-                                                 sizeof(double) * R)[t];
-          xs[t * kJTileLd + rr] = a;
-        }
-        continue;
-      }
+      if (e - b > kHeavyRatings) continue;  // below, by the whole block
       float hrow[S::CPL];
       double rhs;
       joint_accumulate<T, RP>(ycol, yval, other, b, e, R, tiles + (size_t)warp * 32 * S::LD, hrow, rhs);
@@ -325,8 +313,40 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
       }
       if (h == 0 && i < R) xs[i * kJTileLd + rr] = mu * (double)N[row * R + i] + rhs;
     }
+    if (slots && yptr) {
+      const int64_t own = tile + lane * ntiles;
+      unsigned heavy = __ballot_sync(kFull, lane < nr && yptr[own + 1] - yptr[own] > kHeavyRatings);
+      for (; heavy; heavy &= heavy - 1u) {
+        const int rr = __ffs(heavy) - 1;
+        const int64_t row = tile + rr * ntiles;
+        const int64_t b = yptr[row], e = yptr[row + 1];
+        // the row's pieces in order, a thread per entry
+        const int64_t k0 = b / kHeavyRatings, k1 = (e - 1) / kHeavyRatings;
+        const unsigned char* p0 = slots + (2 * k0 + (b % kHeavyRatings ? 1 : 0)) * jslot_bytes(R);
+        const unsigned char* pk = slots + 2 * (k0 + 1) * jslot_bytes(R);  // the pieces after the first
+        const int64_t np = k1 - k0;
+        const size_t step = 2 * jslot_bytes(R);
+        for (int t = threadIdx.x; t < jtri(R) + R; t += kJSolveWarps * 32) {
+          if (t < jtri(R)) {
+            int ti = 0;
+            while (jtri(ti + 1) <= t) ++ti;
+            double a = (double)reinterpret_cast<const float*>(p0)[t];
+#pragma unroll 8
+            for (int64_t k = 0; k < np; ++k) a += (double)reinterpret_cast<const float*>(pk + k * step)[t];
+            Hs[t * kJTileLd + rr] = base[ti * R + (t - jtri(ti))] + a;
+          } else {
+            const int i2 = t - jtri(R);
+            const size_t at = jslot_bytes(R) - sizeof(double) * (R - i2);
+            double a = mu * (double)N[row * R + i2] + *reinterpret_cast<const double*>(p0 + at);
+#pragma unroll 8
+            for (int64_t k = 0; k < np; ++k) a += *reinterpret_cast<const double*>(pk + k * step + at);
+            xs[i2 * kJTileLd + rr] = a;
+          }
+        }
+      }
+    }
     __syncthreads();
-    if (warp == 0 && lane < nr) {
+    if (warp == solver && lane < nr) {
       // Cholesky H = L L^T row by row below the diagonal, then L L^T x = rhs;
       // the diagonal holds 1 / L[j][j].
       double* H = Hs + lane;
@@ -340,7 +360,7 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
           d -= l * l;
         }
         bad |= !(d > 0.0);
-        const double inv = 1.0 / sqrt(fmax(d, 1e-300));
+        const double inv = rsqrt(fmax(d, 1e-300));
         H[(rj + j) * kJTileLd] = inv;
         int m = j + 1;
         for (; m + 4 <= R; m += 4) {  // four rows at a time (independent chains)
@@ -381,7 +401,7 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
     }
     __syncthreads();
     for (int t = threadIdx.x; t < nr * R; t += kJSolveWarps * 32)
-      st_elem(F + 32 * tile * R + t, (float)xs[(t % R) * kJTileLd + t / R]);
+      st_elem(F + (tile + (t / R) * ntiles) * R + t % R, (float)xs[(t % R) * kJTileLd + t / R]);
     __syncthreads();  // before the next 32 rows
   }
 }

@@ -1,5 +1,5 @@
-"""Joint ALS rows with more ratings than one piece (1,024): rows at and around
-that length, starting on and off a piece boundary, next to empty rows, for both
+"""Joint ALS rows with more ratings than one piece (256): rows at and around
+that length and its multiples, starting on and off a piece boundary, next to empty rows, for both
 sides and ranks that fill and do not fill the row solver's layouts."""
 import numpy as np
 import pytest
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("swap", [False, True])
 @pytest.mark.parametrize("R", [1, 5, 8, 12, 16, 24, 32])
 def test_long_rating_rows(R, swap, dtype):
-    counts = [1024, 1025, 0, 2500, 7, 0, 1, 3071, 40] + [3] * 40
+    counts = [1024, 1025, 0, 2500, 7, 0, 1, 3071, 40, 256, 257, 255] + [3] * 40
     users, items, words = len(counts), 3100, 20
     g = torch.Generator().manual_seed(77 + R)
     pairs = torch.cat([torch.stack([torch.full((n,), u), torch.randperm(items, generator=g)[:n]])
