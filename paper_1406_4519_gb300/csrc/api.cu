@@ -7,6 +7,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <vector>
 
 #include "device.cuh"
 #include "internal.h"
@@ -60,6 +61,69 @@ void keep_pool_memory() {
     cudaGetLastError();
   });
 }
+
+namespace {
+
+// Auxiliary streams (with their two events) of destroyed handles, for the next
+// ones: creating and destroying a set takes longer than most of a small build's
+// kernels.  At most kAuxKept sets are kept per device; a set comes back idle.
+struct AuxSet {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+};
+constexpr int kAuxDevices = 64;
+constexpr size_t kAuxKept = 32;
+struct AuxPool {
+  std::mutex lock;
+  std::vector<AuxSet> free;
+};
+AuxPool& aux_pool(int device) {
+  static AuxPool* pools = new AuxPool[kAuxDevices];  // outlives every static destructor
+  return pools[device];
+}
+
+bool aux_take(dfacto_t* h) {
+  AuxSet a;
+  if (h->device >= 0 && h->device < kAuxDevices) {
+    AuxPool& p = aux_pool(h->device);
+    std::lock_guard<std::mutex> g(p.lock);
+    if (!p.free.empty()) {
+      a = p.free.back();
+      p.free.pop_back();
+    }
+  }
+  if (a.stream) {
+    h->aux = a.stream;
+    h->aux_fork = a.fork;
+    h->aux_join = a.join;
+    return true;
+  }
+  return cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&h->aux_fork, cudaEventDisableTiming) == cudaSuccess &&
+         cudaEventCreateWithFlags(&h->aux_join, cudaEventDisableTiming) == cudaSuccess;
+}
+
+void aux_give(dfacto_t* h) {
+  const bool idle = h->aux && cudaStreamSynchronize(h->aux) == cudaSuccess;
+  if (idle && h->aux_fork && h->aux_join && h->device >= 0 && h->device < kAuxDevices) {
+    AuxPool& p = aux_pool(h->device);
+    std::lock_guard<std::mutex> g(p.lock);
+    if (p.free.size() < kAuxKept) {
+      try {
+        p.free.push_back(AuxSet{h->aux, h->aux_fork, h->aux_join});
+        h->aux = nullptr;
+        h->aux_fork = h->aux_join = nullptr;
+        return;
+      } catch (...) {  // no memory for the entry: destroyed below
+      }
+    }
+  }
+  if (h->aux) cudaStreamDestroy(h->aux);
+  if (h->aux_fork) cudaEventDestroy(h->aux_fork);
+  if (h->aux_join) cudaEventDestroy(h->aux_join);
+}
+
+}  // namespace
 
 dfacto_status dalloc(dfacto_t* h, void** p, size_t bytes) {
   *p = nullptr;
@@ -266,12 +330,7 @@ void dfacto_destroy(dfacto_t* h) {
     if (q) cudaFreeAsync(q, h->stream);
   delete[] h->host_scal;
   delete[] h->host_flags;
-  if (h->aux) {
-    cudaStreamSynchronize(h->aux);
-    cudaStreamDestroy(h->aux);
-  }
-  if (h->aux_fork) cudaEventDestroy(h->aux_fork);
-  if (h->aux_join) cudaEventDestroy(h->aux_join);
+  aux_give(h);
   cudaGetLastError();
   delete h;
 }
@@ -319,7 +378,7 @@ dfacto_status dfacto_build(const int32_t* idx, const float* val, int64_t nnz, co
   dfacto_status st = DFACTO_OK;
   const size_t RR = (size_t)R * R;
   const int64_t maxdim = std::max<int64_t>(dims[0], std::max<int64_t>(dims[1], dims[2]));
-  if ((st = dalloc(h, (void**)&h->scal, sizeof(double) * kNumScalars)) != DFACTO_OK) return bail(st);
+  if ((st = dalloc(h, (void**)&h->scal, sizeof(double) * (kNumScalars + 1))) != DFACTO_OK) return bail(st);
   if ((st = dalloc(h, (void**)&h->flags, sizeof(int32_t) * kNumFlags)) != DFACTO_OK) return bail(st);
   if ((st = grow_partials(h, std::max<int64_t>(608 * (int64_t)RR, 4096))) != DFACTO_OK) return bail(st);
   if ((st = dalloc(h, (void**)&h->lambda, sizeof(double) * R)) != DFACTO_OK) return bail(st);
@@ -337,9 +396,7 @@ dfacto_status dfacto_build(const int32_t* idx, const float* val, int64_t nnz, co
     if ((st = dalloc(h, &h->F[m], elem_size(h->dtype) * (size_t)dims[m] * R)) != DFACTO_OK) return bail(st);
     if ((st = dalloc(h, (void**)&h->gram[m], sizeof(double) * RR)) != DFACTO_OK) return bail(st);
   }
-  if (cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&h->aux_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&h->aux_join, cudaEventDisableTiming) != cudaSuccess) {
+  if (!aux_take(h)) {
     cudaGetLastError();
     return bail(DFACTO_ECUDA);
   }
@@ -347,7 +404,7 @@ dfacto_status dfacto_build(const int32_t* idx, const float* val, int64_t nnz, co
   h->host_flags = new (std::nothrow) int32_t[kNumFlags]();
   if (!h->host_scal || !h->host_flags) return bail(DFACTO_ENOMEM);
   cudaStream_t s = h->stream;
-  if (cudaMemsetAsync(h->scal, 0, sizeof(double) * kNumScalars, s) != cudaSuccess) return bail(DFACTO_ECUDA);
+  if (cudaMemsetAsync(h->scal, 0, sizeof(double) * (kNumScalars + 1), s) != cudaSuccess) return bail(DFACTO_ECUDA);
   for (int m = 0; m < 3; ++m)
     if (cudaMemsetAsync(h->F[m], 0, elem_size(h->dtype) * (size_t)dims[m] * R, s) != cudaSuccess)
       return bail(DFACTO_ECUDA);

@@ -107,7 +107,7 @@ struct dfacto_handle {
   double* W = nullptr;                        // [R x R] Gamma^{-1} (FP64)
   double* rr_work = nullptr;                  // [2 R^2 + R] workspace of the R x R solve
   float* W32 = nullptr;                       // [R x R] Gamma^{-1} (FP32)
-  double* scal = nullptr;                     // [kNumScalars]
+  double* scal = nullptr;                     // [kNumScalars], then the row passes' block counter (zero between launches)
   int32_t* flags = nullptr;                   // [kNumFlags]
   double* partials = nullptr;                 // reduction partials
   int64_t partials_cap = 0;                   // doubles

@@ -80,11 +80,57 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan(const int32_t* in, int
   }
 }
 
+// The whole scan by one block of 1024 threads, 16 values each and round: up to
+// kOneBlock values, the time of one of the three launches it saves.
+constexpr int kOneThreads = 1024;
+constexpr int64_t kOneBlock = 4 * 16 * kOneThreads;
+__global__ void __launch_bounds__(kOneThreads) one_block_scan(const int32_t* in, int32_t* out, int64_t n) {
+  constexpr int V = 16;
+  __shared__ int32_t s_warp[kOneThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t run = 0;
+  for (int64_t t0 = 0; t0 < n; t0 += (int64_t)kOneThreads * V) {
+    const int64_t t = t0 + (int64_t)threadIdx.x * V;
+    int32_t x[V];
+    int32_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      x[k] = t + k < n ? in[t + k] : 0;
+      sum += x[k];
+    }
+    int32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    int32_t ofs = run + incl - sum, all = 0;
+    for (int w = 0; w < kOneThreads / 32; ++w) {
+      const int32_t y = s_warp[w];
+      if (w < warp) ofs += y;
+      all += y;
+    }
+    run += all;
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      if (t + k < n) out[t + k] = ofs;
+      ofs += x[k];
+    }
+    __syncthreads();  // s_warp is rewritten next round; in may alias out
+  }
+}
+
 }  // namespace
 
 cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
+  if (ntiles > 1 && n <= kOneBlock) {
+    one_block_scan<<<1, kOneThreads, 0, s>>>(in, out, n); DF_COUNT();
+    return cudaGetLastError();
+  }
   if (ntiles == 1) {
     tile_scan<<<1, kScanThreads, 0, s>>>(in, out, n, nullptr); DF_COUNT();
     return cudaGetLastError();
