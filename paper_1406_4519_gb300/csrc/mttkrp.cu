@@ -18,9 +18,9 @@ constexpr int kWalkWaves = 2;
 constexpr int kAheadCols = 32;  // carry values per lane a warp loads before adding them
 
 // One block per CTA c (grid-stride): if c's last partial run belongs to a row r
-// that starts inside c, add up r's partials from CTAs c .. c_last in CTA order
-// (eight warps take interleaved entries, then their sums are added in warp
-// order) and store N[r, :].  Then all blocks zero the rows without fibers.
+// that starts inside c, add up r's partials from CTAs c .. c_last in a fixed
+// order (eight warps take interleaved entries, a batch of them as a tree, then
+// their FP64 sums are added in warp order) and store N[r, :].  Then all blocks zero the rows without fibers.
 // `bad` (nullable) is set when a carry entry does not name the row it should.
 // CPL = columns per lane (R <= 32 * CPL); a warp keeps 32 / CPL entries in
 // flight, which bounds the time of the longest row (a heavy row of a
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
     const int32_t* __restrict__ carry_row, const float* __restrict__ carry,
     const int64_t* __restrict__ fiber_ptr, const int64_t* __restrict__ nz_ptr, float* __restrict__ out,
     int R, int64_t P, int64_t ncta, int64_t dim_o, int32_t* __restrict__ bad) {
-  __shared__ float part[kFixWarps][128];
+  __shared__ double part[kFixWarps][128];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int64_t c = blockIdx.x; c < ncta; c += gridDim.x) {
     const int k = carry_row[2 * c + 1] >= 0 ? 1 : 0;
@@ -41,9 +41,9 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
     const int64_t re = nz_ptr[fiber_ptr[r + 1]];
     const int64_t clast = (re - 1) / P;
     const int64_t ne = clast - c + 1;
-    float s[CPL];
+    double s[CPL];
 #pragma unroll
-    for (int q = 0; q < CPL; ++q) s[q] = 0.f;
+    for (int q = 0; q < CPL; ++q) s[q] = 0.0;
     // Warp w adds entries w, w + 8, w + 16, ... in that order; kAhead of them
     // are loaded before the adds so that their loads overlap.
     constexpr int kAhead = kAheadCols / CPL;
@@ -59,12 +59,18 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
           t[u][q] = (j < ne && col < R) ? carry[entry * R + col] : 0.f;
         }
       }
-      // Entries past the end hold +0 and are added too (no branch between the
-      // loads and the adds); only the sign of a zero sum can differ.
+      // A tree in FP32 over the batch, then one FP64 add: a heavy row's partials
+      // are the longest chain of its sum, at the full magnitude of the result,
+      // and FP64 instructions are slow (all of them in FP64: 25 us more per mode
+      // of 50M nonzeros).  Entries past the end hold +0 and are added too.
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u)
+      for (int w = kAhead / 2; w > 0; w >>= 1)
 #pragma unroll
-        for (int q = 0; q < CPL; ++q) s[q] += t[u][q];
+        for (int u = 0; u < w; ++u)
+#pragma unroll
+          for (int q = 0; q < CPL; ++q) t[u][q] += t[u + w][q];
+#pragma unroll
+      for (int q = 0; q < CPL; ++q) s[q] += (double)t[0][q];
       if (lane < kAhead) {
         const int64_t j = j0 + (int64_t)lane * kFixWarps;
         if (bad && j > 0 && j < ne && carry_row[2 * (c + j)] != r) atomicOr(bad, 1);
@@ -81,9 +87,9 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
       for (int q = 0; q < CPL; ++q) {
         const int col = lane + 32 * q;
         if (col < R) {
-          float t = 0.f;
-          for (int w = 0; w < kFixWarps; ++w) t += part[w][col];
-          out[(int64_t)r * R + col] = t;
+          double t = part[0][col];
+          for (int w = 1; w < kFixWarps && w < ne; ++w) t += part[w][col];
+          out[(int64_t)r * R + col] = (float)t;
         }
       }
     }
