@@ -444,8 +444,8 @@ dfacto_status dfacto_build(const int32_t* idx, const float* val, int64_t nnz, co
   for (int m = 0; m < 3; ++m) {
     // the walk's own rank and gathered type (padded FP32 copies at a padded rank)
     const int RP = walk_rank(R, opt.vec);
-    h->m[m].cfg = RP != R ? choose_walk(RP, DFACTO_F32, nnz, h->m[m].nfib, opt.seg_nnz, 0)
-                          : choose_walk(R, h->dtype, nnz, h->m[m].nfib, opt.seg_nnz, opt.vec);
+    h->m[m].cfg = RP != R ? choose_walk(RP, DFACTO_F32, nnz, h->m[m].nfib, walk_segment(h->dtype, opt.seg_nnz), 0)
+                          : choose_walk(R, h->dtype, nnz, h->m[m].nfib, walk_segment(h->dtype, opt.seg_nnz), opt.vec);
     if (opt.walk > 0) {
       h->m[m].cfg.kernel = opt.walk;
     }

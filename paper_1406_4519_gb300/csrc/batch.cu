@@ -303,7 +303,7 @@ dfacto_status batch_mttkrp_issue(dfacto_batch* b, int mode, cudaStream_t s,
     const int64_t P = (int64_t)C.segs() * C.cfg.seg;
     DB_CUDA(b, launch_mttkrp_fixup(C.carry_row, C.carry, C.m[mode].fiber_ptr, C.m[mode].nz_ptr,
                                    C.m[mode].N, C.R, P, C.nnz > 0 ? C.ncta() : 0, C.m[mode].dim_o,
-                                   b->d_bad, s));
+                                   b->d_bad, C.dtype == DFACTO_BF16, s));
   }
   return DFACTO_OK;
 }
@@ -639,7 +639,7 @@ dfacto_status dfacto_batch_create(dfacto_t* const* jobs, int32_t n, const dfacto
     for (int mode = 0; mode < 3; ++mode)
       if ((st = build_class_mode(b, C, mode)) != DFACTO_OK) return bail(st);
     // Walk configuration: the single-tensor default, then (optionally) tuned.
-    C.cfg = choose_walk(C.R, C.dtype, C.nnz, C.m[0].nfib, 0, 0);
+    C.cfg = choose_walk(C.R, C.dtype, C.nnz, C.m[0].nfib, walk_segment(C.dtype, 0), 0);
     C.cfg.kernel = 2;
     int min_seg = C.cfg.seg;
     int64_t min_P = (int64_t)C.segs() * C.cfg.seg;

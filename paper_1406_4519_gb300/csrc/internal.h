@@ -177,6 +177,7 @@ dfacto_status ensure_segments(dfacto_t* h, int mode);
 
 // ---- MTTKRP (mttkrp*.cu) --------------------------------------------------
 WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, int vec_opt);
+int walk_segment(int dtype, int seg_opt);
 // Rank the MTTKRP walk runs at: R, or R rounded up to a multiple of four (the
 // factors then gathered from zero-padded FP32 copies) when R > 2 is not one
 // and no lane width was asked for.

@@ -2,6 +2,7 @@
 // fix-up kernel that finishes rows spanning several CTAs and zero-fills rows
 // with no nonzeros.
 #include <algorithm>
+#include <type_traits>
 
 #include "mttkrp.cuh"
 
@@ -20,17 +21,20 @@ constexpr int kAheadCols = 32;  // carry values per lane a warp loads before add
 // One block per CTA c (grid-stride): if c's last partial run belongs to a row r
 // that starts inside c, add up r's partials from CTAs c .. c_last in a fixed
 // order (eight warps take interleaved entries, a batch of them as a tree, then
-// their FP64 sums are added in warp order) and store N[r, :].  Then all blocks zero the rows without fibers.
+// their FP64 sums are added in warp order) and store N[r, :].  Then all blocks
+// zero the rows without fibers.  With SERIAL the entries are added one after
+// another in FP32: the order of handles with BF16 factors (see walk_segment).
 // `bad` (nullable) is set when a carry entry does not name the row it should.
 // CPL = columns per lane (R <= 32 * CPL); a warp keeps 32 / CPL entries in
 // flight, which bounds the time of the longest row (a heavy row of a
 // power-law mode spans over a thousand CTAs).
-template <int CPL>
+template <int CPL, bool SERIAL>
 __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
     const int32_t* __restrict__ carry_row, const float* __restrict__ carry,
     const int64_t* __restrict__ fiber_ptr, const int64_t* __restrict__ nz_ptr, float* __restrict__ out,
     int R, int64_t P, int64_t ncta, int64_t dim_o, int32_t* __restrict__ bad) {
-  __shared__ double part[kFixWarps][128];
+  using Acc = std::conditional_t<SERIAL, float, double>;
+  __shared__ Acc part[kFixWarps][128];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int64_t c = blockIdx.x; c < ncta; c += gridDim.x) {
     const int k = carry_row[2 * c + 1] >= 0 ? 1 : 0;
@@ -41,9 +45,9 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
     const int64_t re = nz_ptr[fiber_ptr[r + 1]];
     const int64_t clast = (re - 1) / P;
     const int64_t ne = clast - c + 1;
-    double s[CPL];
+    Acc s[CPL];
 #pragma unroll
-    for (int q = 0; q < CPL; ++q) s[q] = 0.0;
+    for (int q = 0; q < CPL; ++q) s[q] = 0;
     // Warp w adds entries w, w + 8, w + 16, ... in that order; kAhead of them
     // are loaded before the adds so that their loads overlap.
     constexpr int kAhead = kAheadCols / CPL;
@@ -63,14 +67,21 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
       // are the longest chain of its sum, at the full magnitude of the result,
       // and FP64 instructions are slow (all of them in FP64: 25 us more per mode
       // of 50M nonzeros).  Entries past the end hold +0 and are added too.
+      if constexpr (SERIAL) {
 #pragma unroll
-      for (int w = kAhead / 2; w > 0; w >>= 1)
+        for (int u = 0; u < kAhead; ++u)
 #pragma unroll
-        for (int u = 0; u < w; ++u)
+          for (int q = 0; q < CPL; ++q) s[q] += t[u][q];
+      } else {
 #pragma unroll
-          for (int q = 0; q < CPL; ++q) t[u][q] += t[u + w][q];
+        for (int w = kAhead / 2; w > 0; w >>= 1)
 #pragma unroll
-      for (int q = 0; q < CPL; ++q) s[q] += (double)t[0][q];
+          for (int u = 0; u < w; ++u)
+#pragma unroll
+            for (int q = 0; q < CPL; ++q) t[u][q] += t[u + w][q];
+#pragma unroll
+        for (int q = 0; q < CPL; ++q) s[q] += (double)t[0][q];
+      }
       if (lane < kAhead) {
         const int64_t j = j0 + (int64_t)lane * kFixWarps;
         if (bad && j > 0 && j < ne && carry_row[2 * (c + j)] != r) atomicOr(bad, 1);
@@ -87,7 +98,7 @@ __global__ void __launch_bounds__(kFixThreads) mttkrp_fixup(
       for (int q = 0; q < CPL; ++q) {
         const int col = lane + 32 * q;
         if (col < R) {
-          double t = part[0][col];
+          Acc t = part[0][col];
           for (int w = 1; w < kFixWarps && w < ne; ++w) t += part[w][col];
           out[(int64_t)r * R + col] = (float)t;
         }
@@ -190,21 +201,30 @@ cudaError_t pad_factor_rows(const void* src, int src_dtype, int64_t rows, int R,
 
 cudaError_t launch_mttkrp_fixup(const int32_t* carry_row, const float* carry,
                                 const int64_t* fiber_ptr, const int64_t* nz_ptr, float* out, int R,
-                                int64_t P, int64_t ncta, int64_t dim_o, int32_t* bad,
+                                int64_t P, int64_t ncta, int64_t dim_o, int32_t* bad, bool serial,
                                 cudaStream_t s) {
   const int64_t zero_blocks = (dim_o + kFixThreads - 1) / kFixThreads;
-  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(std::max(ncta, zero_blocks), 152 * 16));
-  if (R <= 32)
-    mttkrp_fixup<1><<<(unsigned)blocks, kFixThreads, 0, s>>>(carry_row, carry, fiber_ptr, nz_ptr, out,
-                                                              R, P, ncta, dim_o, bad);
-  else if (R <= 64)
-    mttkrp_fixup<2><<<(unsigned)blocks, kFixThreads, 0, s>>>(carry_row, carry, fiber_ptr, nz_ptr, out,
-                                                              R, P, ncta, dim_o, bad);
-  else
-    mttkrp_fixup<kMaxColsPerLane><<<(unsigned)blocks, kFixThreads, 0, s>>>(
-        carry_row, carry, fiber_ptr, nz_ptr, out, R, P, ncta, dim_o, bad);
+  const unsigned blocks =
+      (unsigned)std::max<int64_t>(1, std::min<int64_t>(std::max(ncta, zero_blocks), 152 * 16));
+  auto go = [&](auto kernel) {
+    kernel<<<blocks, kFixThreads, 0, s>>>(carry_row, carry, fiber_ptr, nz_ptr, out, R, P, ncta, dim_o, bad);
+  };
+  if (R <= 32) serial ? go(mttkrp_fixup<1, true>) : go(mttkrp_fixup<1, false>);
+  else if (R <= 64) serial ? go(mttkrp_fixup<2, true>) : go(mttkrp_fixup<2, false>);
+  else serial ? go(mttkrp_fixup<kMaxColsPerLane, true>) : go(mttkrp_fixup<kMaxColsPerLane, false>);
   DF_COUNT();
   return cudaGetLastError();
+}
+
+// Segment length of a handle whose factors are stored as `dtype`, if none is
+// asked for (0: by size).  BF16 factors round every updated entry to eight bits,
+// so a last-bit change of a sum now and then moves an entry by 2^-9 and the next
+// mode's weights by up to 1e-3; their sums keep one order at every size
+// (segments of 128 and a serial fix-up), so that results do not depend on how
+// the work is split.  5M uniform nonzeros, R = 16: 363 us for three modes, 319
+// with segments by size.
+int walk_segment(int dtype, int seg_opt) {
+  return seg_opt > 0 ? seg_opt : dtype == DFACTO_BF16 ? 128 : 0;
 }
 
 WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, int vec_opt) {
@@ -329,7 +349,7 @@ dfacto_status walk_rows(dfacto_t* h, int mode, float* wout) {
     if (e != cudaSuccess) return cuda_fail(h, e, "mttkrp_walk launch");
   }
   DF_CUDA(h, launch_mttkrp_fixup(h->carry_row, h->carry, M.fiber_ptr, M.nz_ptr, wout, RP, P, ncta,
-                                 M.dim_o, h->flags + kFlagInternal, h->stream));
+                                 M.dim_o, h->flags + kFlagInternal, h->dtype == DFACTO_BF16, h->stream));
   return DFACTO_OK;
 }
 

@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) mttkrp_walk(const MttkrpParam
 // R = 32), so what counts is how many are in flight and how few instructions
 // stand between two rounds: the earlier form of this walk parked the fiber sums
 // in shared memory and folded them in a second, dependent round of loads (18
-// warp instructions per nonzero, now 9).  Per mode of 50M power-law nonzeros,
+// warp instructions per nonzero, now 8).  Per mode of 50M power-law nonzeros,
 // before and now: R = 32 1.05 and 0.85 ms, R = 16 0.64 and 0.52, R = 8 0.59 and
 // 0.40, R = 32 with BF16 factors 1.04 and 0.56.  Slower here: the streams
 // staged in shared memory by cp.async (0.87 ms at R = 32, 12 instructions), the
@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, (Walk2Shape<T, VEC, G>::MIN_B
 // (build.cu), shared with the allocation-free entry point.
 cudaError_t launch_mttkrp_fixup(const int32_t* carry_row, const float* carry,
                                 const int64_t* fiber_ptr, const int64_t* nz_ptr, float* out, int R,
-                                int64_t P, int64_t ncta, int64_t dim_o, int32_t* bad,
+                                int64_t P, int64_t ncta, int64_t dim_o, int32_t* bad, bool serial,
                                 cudaStream_t s);
 cudaError_t launch_segment_starts(const int64_t* nz_ptr, int64_t nfib, int64_t nseg, int64_t seg,
                                   int32_t* seg_fib, cudaStream_t s);
