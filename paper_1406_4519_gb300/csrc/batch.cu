@@ -334,13 +334,23 @@ dfacto_status time_class(dfacto_batch* b, int k, int reps, double* ms) {
 
 // Candidate walk configurations of class C: columns per lane (the R tile of a
 // lane) and nonzeros per segment; the lanes per segment follow from R.
+//
+// A BF16 class has one: its shape sets the order of its sums, and BF16 storage
+// turns a last bit of a sum into 2^-9 of a factor entry now and then, so a shape
+// chosen by time would make the factors of a batch differ between two creations.
+// Segments of 64 with four columns per lane (eight where four would take more
+// than four lanes) are what timing mostly chose when every BF16 class was timed;
+// ranks without such a shape keep the default.  48 uneven jobs, ranks 8, 16, 32
+// (32M nonzeros): 1.59 ms for the three modes' walks, 1.49 with segments of 128.
 std::vector<WalkCfg> candidates(const BatchClass& C) {
   std::vector<WalkCfg> out;
   for (int vec : {4, 8}) {
     if (C.R % vec != 0) continue;
     const int G = next_pow2((C.R + vec - 1) / vec);
     if (G > 32 || (vec == 8 && G > 16)) continue;
+    if (C.dtype == DFACTO_BF16 && (C.R < 8 || C.R > 32 || vec != (C.R > 16 && C.R % 8 == 0 ? 8 : 4))) continue;
     for (int seg : kTuneSegs) {
+      if (C.dtype == DFACTO_BF16 && seg != kTuneSegs[0]) continue;
       WalkCfg c;
       c.vec = vec;
       c.G = G;
@@ -355,7 +365,7 @@ std::vector<WalkCfg> candidates(const BatchClass& C) {
 dfacto_status autotune_class(dfacto_batch* b, int k) {
   BatchClass& C = b->cls[k];
   const std::vector<WalkCfg> cands = candidates(C);
-  if (cands.size() < 2 || C.nnz == 0) return DFACTO_OK;
+  if (cands.empty() || C.nnz == 0) return DFACTO_OK;
   WalkCfg best = C.cfg;
   double best_ms = 1e300;
   for (const WalkCfg& c : cands) {

@@ -219,10 +219,11 @@ cudaError_t launch_mttkrp_fixup(const int32_t* carry_row, const float* carry,
 // Segment length of a handle whose factors are stored as `dtype`, if none is
 // asked for (0: by size).  BF16 factors round every updated entry to eight bits,
 // so a last-bit change of a sum now and then moves an entry by 2^-9 and the next
-// mode's weights by up to 1e-3; their sums keep one order at every size
-// (segments of 128 and a serial fix-up), so that results do not depend on how
-// the work is split.  5M uniform nonzeros, R = 16: 363 us for three modes, 319
-// with segments by size.
+// mode's weights by up to 1e-3.  A handle with BF16 factors therefore keeps one
+// segment length and the fix-up's order of addition (SERIAL) at every size; a
+// batch cuts the concatenated nonzeros of its jobs, at lengths of its own
+// (batch.cu), so a job's sums are added in another order there.  5M uniform
+// nonzeros, R = 16: 363 us for three modes, 319 with segments by size.
 int walk_segment(int dtype, int seg_opt) {
   return seg_opt > 0 ? seg_opt : dtype == DFACTO_BF16 ? 128 : 0;
 }
