@@ -347,7 +347,7 @@ std::vector<WalkCfg> candidates(const BatchClass& C) {
   for (int vec : {4, 8}) {
     if (C.R % vec != 0) continue;
     const int G = next_pow2((C.R + vec - 1) / vec);
-    if (G > 32 || (vec == 8 && G > 16)) continue;
+    if (vec == 4 ? G < 2 || G > 8 : G > 4) continue;  // other ranks keep the default
     if (C.dtype == DFACTO_BF16 && (C.R < 8 || C.R > 32 || vec != (C.R > 16 && C.R % 8 == 0 ? 8 : 4))) continue;
     for (int seg : kTuneSegs) {
       if (C.dtype == DFACTO_BF16 && seg != kTuneSegs[0]) continue;

@@ -11,10 +11,10 @@ namespace {
 
 constexpr int kFixThreads = 256;
 constexpr int kFixWarps = kFixThreads / 32;
-// Waves of walk CTAs (152 SMs, two resident) below which segments get shorter:
-// two, measured against one and four (5M uniform nonzeros, R = 16, BF16: 96 us
-// per mode against 106 and 105; the same within 1% on 1M to 60M power-law
-// nonzeros).
+// Waves of walk CTAs (152 SMs, two resident) below which segments get shorter.
+// Two, against one and four: 121, 124 and 121 us per mode of 5M uniform nonzeros
+// at R = 4 (segments of 32, 64, 32), 114, 114 and 112 at R = 16 (128, 128, 64);
+// eight other sizes of 10,000 to 5M nonzeros within 3%.
 constexpr int kWalkWaves = 2;
 constexpr int kAheadCols = 32;  // carry values per lane a warp loads before adding them
 
@@ -244,16 +244,16 @@ WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, in
   c.vec = vec;
   c.G = G;
   c.kernel = 2;  // fiber ends from the end bitmask (faster on every measured shape)
-  
-  // Segment length: a CTA's fixed cost (its first dependent loads and the merge
-  // of its partial rows) is paid per segment, so long segments are better as
-  // long as the CTAs fill the GPU kWalkWaves times over (50M power-law
-  // nonzeros, R = 16: 530 us per mode with segments of 128, 514 with 256; 10,000
-  // uniform nonzeros, R = 10: 39 us with 128, 29 with 32).
+
+  // Segment length: 128, or shorter where the CTAs would not fill the GPU
+  // kWalkWaves times over (27,773 nonzeros, R = 24: 57 us for three modes with
+  // 32, 108 with 128).  Never longer: a segment is the longest FP32 chain of a
+  // row's sum (50M power-law nonzeros, R = 32: 860 us per mode with 256 and 901
+  // with 128, but 2.2e-7 from 64 bits and 1.8e-7).
   const int segs = kWalkWarps * (32 / G);
   int seg = seg_opt;
   if (seg <= 0) {
-    seg = 256;
+    seg = 128;
     while (seg > 32 && nnz < (int64_t)segs * seg * kWalkWaves * 152 * 2) seg >>= 1;
   }
   seg = std::max(32, (seg + 31) / 32 * 32);

@@ -1,7 +1,6 @@
 // noalloc.cu -- dfacto_mttkrp_noalloc: the MTTKRP of one mode for callers that
 // must not allocate device memory.  Everything it needs besides the caller's
 // inputs and output lives in one fixed device array defined in this file.
-#include <algorithm>
 #include <mutex>
 
 #include "mttkrp.cuh"
@@ -79,10 +78,7 @@ extern "C" dfacto_status dfacto_mttkrp_noalloc(const dfacto_csr_view* csr, const
   // Eight columns per lane where R allows it (R a multiple of 8: R / 8 lanes
   // per segment), fewer otherwise; the walk shape fixes the scratch per
   // nonzero stated in the header.
-  // Segments are at most 128 nonzeros, so that the fixed scratch takes and
-  // refuses the sizes stated there.
-  WalkCfg cfg = choose_walk(R, DFACTO_F32, nnz, nfib, 0, 8);
-  cfg.seg = std::min(cfg.seg, 128);
+  const WalkCfg cfg = choose_walk(R, DFACTO_F32, nnz, nfib, 0, 8);
   const int segs = kWalkWarps * (32 / cfg.G);
   const int64_t P = (int64_t)segs * cfg.seg;
   const int64_t ncta = (nnz + P - 1) / P;

@@ -47,3 +47,17 @@ def test_bf16_batches_of_the_same_jobs_agree_bit_for_bit():
         assert got[0][1] == got[1][1]
         for f0, f1 in zip(got[0][0], got[1][0]):
             assert all(torch.equal(x, y) for x, y in zip(f0, f1)), R
+
+
+def test_default_segments_hold_no_longer_chain_than_128():
+    # enough nonzeros that a rule by size alone would take longer segments
+    dims, R = [60000, 50000, 40000], 32
+    idx, val = synth.uniform_tensor(dims, 12000000, seed=77, device="cuda")
+    F = synth.normal_factors(dims, R, seed=78, device="cuda")
+    got = []
+    for seg in (0, 128):
+        t = dfacto.Tensor(idx, val, dims, rank=R, seg_nnz=seg)
+        assert max(dfacto.dfacto_get_info(t.h).seg_nnz) <= 128
+        t.set_factors(F)
+        got.append([t.mttkrp(m) for m in range(3)])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
