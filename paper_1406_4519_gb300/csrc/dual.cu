@@ -181,6 +181,21 @@ __global__ void __launch_bounds__(kWalkWarps * 32) dual_walk(const DualParams a)
 // without spills; four spill and take 5% longer, two at 80 registers 20%).
 constexpr int kDualGathers = 2;
 
+// s w.
+template <int VEC>
+__device__ __forceinline__ Cols<VEC> scale_cols(float s, const Cols<VEC>& w) {
+  Cols<VEC> o;
+  if constexpr (VEC == 1) {
+    o.p[0] = s * w.p[0];
+  } else {
+    uint64_t ss;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(ss) : "f"(s));
+#pragma unroll
+    for (int e = 0; e < VEC / 2; ++e) asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(o.p[e]) : "l"(ss), "l"(w.p[e]));
+  }
+  return o;
+}
+
 // If `on` is nonzero: u1 += c vG, u2 += (sC g) vB, u3 += (sC g) vG, vB = vG = 0.
 template <int VEC>
 __device__ __forceinline__ void fold_dual_if(uint32_t on, const Cols<VEC>& cf, const Cols<VEC>& gcf, float sC,
@@ -329,7 +344,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) dual_walk2(const DualParam
               }
             }
             axpy_cols<VEC>(xu, bi[uu].get(), vB);
-            axpy_cols<VEC>(xu * sB, gb[uu].get(), vG);  // a power of two scales exactly
+            // the gradient is scaled, not x: x sB can leave the range of FP32
+            axpy_cols<VEC>(xu, scale_cols<VEC>(sB, gb[uu].get()), vG);
             fold_dual_if<VEC>(e4 & (1u << uu), ci[uu].get(), gc[uu].get(), sC, vB, vG, u1, u2, u3);
           }
         }
