@@ -7,10 +7,10 @@
 #include <cstring>
 #include <mutex>
 #include <new>
-#include <vector>
 
 #include "device.cuh"
 #include "internal.h"
+#include "kept_sets.h"
 #include "smem_optin.h"
 
 namespace dfacto {
@@ -65,34 +65,50 @@ void keep_pool_memory() {
 namespace {
 
 // Auxiliary streams (with their two events) of destroyed handles, for the next
-// ones: creating and destroying a set takes longer than most of a small build's
-// kernels.  At most kAuxKept sets are kept per device; a set comes back idle.
+// ones of the same context: creating and destroying a set takes longer than most
+// of a small build's kernels.  A set comes back idle.
 struct AuxSet {
   cudaStream_t stream = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
 };
-constexpr int kAuxDevices = 64;
-constexpr size_t kAuxKept = 32;
-struct AuxPool {
-  std::mutex lock;
-  std::vector<AuxSet> free;
-};
-AuxPool& aux_pool(int device) {
-  static AuxPool* pools = new AuxPool[kAuxDevices];  // outlives every static destructor
-  return pools[device];
+
+KeptSets<AuxSet>* aux_sets() {
+  static auto* sets = new (std::nothrow) KeptSets<AuxSet>();  // outlives every static destructor
+  return sets;
+}
+
+// Id of the calling thread's current context; 0 (nothing is kept) if the driver
+// does not tell.  The driver's entry points come through the runtime, so that
+// the library does not link libcuda.
+uint64_t context_id() {
+  using GetCurrent = int (*)(void**);
+  using GetId = int (*)(void*, unsigned long long*);
+  struct Driver {
+    GetCurrent current = nullptr;
+    GetId id = nullptr;
+    Driver() {
+      cudaDriverEntryPointQueryResult r;
+      void *c = nullptr, *i = nullptr;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &c, 12000, cudaEnableDefault, &r) == cudaSuccess &&
+          cudaGetDriverEntryPointByVersion("cuCtxGetId", &i, 12000, cudaEnableDefault, &r) == cudaSuccess) {
+        current = reinterpret_cast<GetCurrent>(c);
+        id = reinterpret_cast<GetId>(i);
+      } else {
+        cudaGetLastError();
+      }
+    }
+  };
+  static const Driver drv;
+  void* ctx = nullptr;
+  unsigned long long id = 0;
+  if (!drv.current || !drv.id || drv.current(&ctx) != 0 || !ctx || drv.id(ctx, &id) != 0) return 0;
+  return id;
 }
 
 bool aux_take(dfacto_t* h) {
   AuxSet a;
-  if (h->device >= 0 && h->device < kAuxDevices) {
-    AuxPool& p = aux_pool(h->device);
-    std::lock_guard<std::mutex> g(p.lock);
-    if (!p.free.empty()) {
-      a = p.free.back();
-      p.free.pop_back();
-    }
-  }
-  if (a.stream) {
+  h->context = context_id();
+  if (h->context && aux_sets() && aux_sets()->take(h->context, &a)) {
     h->aux = a.stream;
     h->aux_fork = a.fork;
     h->aux_join = a.join;
@@ -105,19 +121,9 @@ bool aux_take(dfacto_t* h) {
 
 void aux_give(dfacto_t* h) {
   const bool idle = h->aux && cudaStreamSynchronize(h->aux) == cudaSuccess;
-  if (idle && h->aux_fork && h->aux_join && h->device >= 0 && h->device < kAuxDevices) {
-    AuxPool& p = aux_pool(h->device);
-    std::lock_guard<std::mutex> g(p.lock);
-    if (p.free.size() < kAuxKept) {
-      try {
-        p.free.push_back(AuxSet{h->aux, h->aux_fork, h->aux_join});
-        h->aux = nullptr;
-        h->aux_fork = h->aux_join = nullptr;
-        return;
-      } catch (...) {  // no memory for the entry: destroyed below
-      }
-    }
-  }
+  if (idle && h->aux_fork && h->aux_join && h->context && aux_sets() &&
+      aux_sets()->give(h->context, AuxSet{h->aux, h->aux_fork, h->aux_join}))
+    return;
   if (h->aux) cudaStreamDestroy(h->aux);
   if (h->aux_fork) cudaEventDestroy(h->aux_fork);
   if (h->aux_join) cudaEventDestroy(h->aux_join);

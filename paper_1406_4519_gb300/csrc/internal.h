@@ -83,6 +83,7 @@ struct dfacto_handle {
   cudaStream_t aux = nullptr;        // Gamma^{-1} beside the MTTKRP (created at build)
   cudaEvent_t aux_fork = nullptr;
   cudaEvent_t aux_join = nullptr;
+  uint64_t context = 0;  // id of the context aux belongs to
   int device = 0;
   int32_t dims[3] = {0, 0, 0};
   int64_t nnz = 0;
