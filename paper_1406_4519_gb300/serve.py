@@ -79,16 +79,23 @@ class JobState:
 
 
 def footprint_bytes(dims: Sequence[int], nnz: int, rank: int, factor_bytes: int) -> int:
-    """Upper estimate of the device bytes a job holds while it is served: the
-    CSR copies of its three modes twice (the job's own and the batch's
-    concatenated copy; per mode 8 bytes per nonzero for (index, value), at most
-    one fiber per nonzero at 16 bytes, 8 bytes per row pointer, end bits), the
-    factors (own and pooled), the MTTKRP outputs, and the row-pass buffers."""
+    """Upper estimate of the device bytes a job holds while it is served, in a
+    batch or alone, whichever is more.  A CSR copy has per mode 8 bytes per
+    nonzero for (index, value), at most one fiber per nonzero at 16 bytes, 8
+    bytes per row pointer, two bits per nonzero (fiber ends, row starts) and a
+    segment start per 32 nonzeros.  In a batch: the job's own copy and the
+    batch's, the factors (own and pooled), the MTTKRP outputs and the row-pass
+    buffers.  Alone, at a rank that the walk pads to a multiple of four: the
+    padded copies of the factors and of the MTTKRP output."""
     sd = sum(int(d) for d in dims)
-    csr = 3 * (8 * nnz + 16 * nnz + nnz // 8 + 4 * nnz // 32) + 8 * (sd + 3)
+    top = max(int(d) for d in dims)
+    csr = 3 * (8 * nnz + 16 * nnz + 2 * (nnz // 8) + 4 * nnz // 32) + 8 * (sd + 3)
     factors = factor_bytes * rank * sd
-    rows = 4 * rank * sd + 2 * 4 * rank * max(dims)
-    return 2 * csr + 2 * factors + rows + (1 << 20)
+    own = 2 * 4 * rank * top
+    batched = 2 * csr + 2 * factors + 4 * rank * sd + own
+    padded = (rank + 3) // 4 * 4 if rank > 2 else rank
+    alone = csr + factors + own + (4 * padded * (sd + top) if padded != rank else 0)
+    return max(batched, alone) + (1 << 20)
 
 
 def converged(fits: Sequence[float], tol: float, relative: bool = True) -> bool:
