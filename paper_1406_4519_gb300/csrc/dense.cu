@@ -1297,6 +1297,15 @@ __device__ __forceinline__ float* row_pass_tile(const float* __restrict__ M, int
   return tile;
 }
 
+// Zero the padding columns R .. ld - 1 of the thread's row of a tile.  N's are not
+// always zero: where a nonzero's value is infinite the walk's are NaN (infinity
+// times the padded factor's zero), and a row's sums over its columns would take
+// that up.
+template <int LD>
+__device__ __forceinline__ void tile_zero_pad(float* __restrict__ tile, int R, int ld) {
+  for (int c = R; c < ld; ++c) tile[threadIdx.x * LD + c] = 0.f;
+}
+
 // Tile rows (already rounded to T) back to rows [t0, t0 + nt) of an R-column
 // matrix in storage type T, with coalesced 16-byte stores where the layout
 // allows (FP32: R % 4 == 0; BF16: R % 8 == 0).
@@ -1541,8 +1550,10 @@ __device__ __forceinline__ void colnorm_rows_tc(const float* __restrict__ N, int
   for (int64_t t0 = r0; t0 < r1; t0 += kT, buf ^= 1) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    const float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
+    float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
+    tile_zero_pad<LD>(tile, R, ldN);
+    __syncwarp();  // a warp takes its own 32 rows
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
       const int m0 = 32 * warp + 16 * mt;
@@ -1618,6 +1629,8 @@ __device__ __forceinline__ void scale_store_rows_tc(const float* __restrict__ N,
     __syncthreads();
     float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
+    tile_zero_pad<LD>(tile, R, ldN);
+    __syncwarp();  // a warp takes its own 32 rows
     float ip32 = 0.f;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
@@ -1711,9 +1724,10 @@ __device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N, i
   for (int64_t t0 = r0; t0 < r1; t0 += kT, buf ^= 1) {
     const int nt = (int)min((int64_t)kT, r1 - t0);
     __syncthreads();
-    const float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
+    float* tile = row_pass_tile<LD>(N, t0, r1, ldN, tiles, buf);
     __syncthreads();
     if ((int)threadIdx.x < nt) {
+      tile_zero_pad<LD>(tile, R, ldN);
       float n[RT];
 #pragma unroll
       for (int c4 = 0; c4 < RT / 4; ++c4) {
@@ -1803,6 +1817,7 @@ __device__ __forceinline__ void scale_store_rows_body(const float* __restrict__ 
     float ip32 = 0.f;
     float* trow = tile + threadIdx.x * LD;
     if ((int)threadIdx.x < nt) {
+      tile_zero_pad<LD>(tile, R, ldN);
       float n[RT];
 #pragma unroll
       for (int c4 = 0; c4 < RT / 4; ++c4) {
@@ -1932,6 +1947,7 @@ __device__ __forceinline__ void gd_rows_tc(const float* __restrict__ N, int ldN,
         tF[threadIdx.x * LD + c] = 0.f;
       }
     }
+    tile_zero_pad<LD>(tN, R, ldN);
     __syncwarp();
     float af[3] = {0.f, 0.f, 0.f};
 #pragma unroll
@@ -2003,6 +2019,7 @@ __global__ void __launch_bounds__(kT, 2) gd_rows(const float* __restrict__ N, in
     __syncthreads();
     float af[3] = {0.f, 0.f, 0.f};
     if ((int)threadIdx.x < nt) {
+      tile_zero_pad<LD>(tN, R, ldN);
       float* nrow = tN + threadIdx.x * LD;
       float f[RT];
 #pragma unroll
