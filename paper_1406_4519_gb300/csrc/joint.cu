@@ -292,9 +292,6 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
   float* tiles = reinterpret_cast<float*>(jsm + (((size_t)(jtri(R) + R) * kJTileLd + 1) & ~(size_t)1));
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane % RP, h = lane / RP;
   const int64_t ntiles = (rows + 31) / 32;
-  // blocks that share an SM solve on different warp schedulers (each retires
-  // half an FP64 lane per clock)
-  const int solver = (blockIdx.x / 152) % kJSolveWarps;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     // rows tile, tile + ntiles, ...: neighbouring rows, which rate alike where
     // labels are ordered by use, go to different blocks
@@ -346,7 +343,7 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
       }
     }
     __syncthreads();
-    if (warp == solver && lane < nr) {
+    if (warp == 0 && lane < nr) {
       // Cholesky H = L L^T row by row below the diagonal, then L L^T x = rhs;
       // the diagonal holds 1 / L[j][j].
       double* H = Hs + lane;
