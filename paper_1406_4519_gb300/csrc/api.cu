@@ -237,6 +237,7 @@ dfacto_status grow_partials(dfacto_t* h, int64_t n) {
 }
 
 dfacto_status convert_factor_in(dfacto_t* h, int m, const void* src, int src_dtype) {
+  note_capture(h);
   const int64_t n = (int64_t)h->dims[m] * h->R;
   const void* dsrc = src;
   void* tmp = nullptr;

@@ -121,6 +121,9 @@ struct dfacto_handle {
   // the output [max dim x walk rank] (all lazy)
   float* pad_F[3] = {nullptr, nullptr, nullptr};
   bool pad_valid[3] = {false, false, false};
+  // a call was recorded into the caller's CUDA graph: a replay changes factors, or
+  // finds them changed, without the host's knowledge, so pad_valid tells nothing
+  bool recorded = false;
   float* pad_out = nullptr;
   // the line search's trilinear pass at such a rank: the gradients as padded
   // FP32 rows [(dims[0] + dims[1] + dims[2]) x walk rank] (lazy)
@@ -190,6 +193,8 @@ dfacto_status mttkrp_launch(dfacto_t* h, int mode, float* out);
 // The MTTKRP into the handle's own buffer: *N gets its rows of *ld columns (ld is
 // the walk rank; columns past R are zero).
 dfacto_status mttkrp_rows(dfacto_t* h, int mode, const float** N, int* ld);
+// Sets h->recorded if the handle's stream is being captured.
+void note_capture(dfacto_t* h);
 // Factor m's padded copy pad_F[m] is up to date afterwards (walk rank != R).
 dfacto_status ensure_padded(dfacto_t* h, int m);
 

@@ -261,10 +261,19 @@ WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, in
   return c;
 }
 
-// The padded FP32 copy of factor m (rank RP), made when the factor changed.
+void note_capture(dfacto_t* h) {
+  if (h->recorded) return;
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &c) != cudaSuccess) cudaGetLastError();
+  else h->recorded = c != cudaStreamCaptureStatusNone;
+}
+
+// The padded FP32 copy of factor m (rank RP), made when the factor changed, and
+// at every call once a call on the handle was recorded into a graph.
 dfacto_status ensure_padded(dfacto_t* h, int m) {
   const int RP = walk_rank(h->R, h->opt.vec);
-  if (h->pad_valid[m]) return DFACTO_OK;
+  note_capture(h);
+  if (h->pad_valid[m] && !h->recorded) return DFACTO_OK;
   dfacto_status st;
   if (!h->pad_F[m] &&
       (st = dalloc(h, reinterpret_cast<void**>(&h->pad_F[m]), sizeof(float) * (size_t)h->dims[m] * RP)) != DFACTO_OK)
