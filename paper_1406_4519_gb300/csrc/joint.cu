@@ -276,6 +276,35 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_heavy(
   }
 }
 
+// The pieces of the heavy row with ratings [b, e), added in order: entry (ti, tj)
+// of the lower triangle to tri(ti, tj, sum) and entry ti of the right side to
+// rhs(ti, sum), a thread per entry (thread t of n).
+template <class Tri, class Rhs>
+__device__ __forceinline__ void add_pieces(const unsigned char* __restrict__ slots, int64_t b, int64_t e, int R,
+                                           int t0, int n, Tri&& tri, Rhs&& rhs) {
+  const int64_t k0 = b / kHeavyRatings, np = (e - 1) / kHeavyRatings - k0;
+  const unsigned char* p0 = slots + (2 * k0 + (b % kHeavyRatings ? 1 : 0)) * jslot_bytes(R);
+  const unsigned char* pk = slots + 2 * (k0 + 1) * jslot_bytes(R);  // the pieces after the first
+  const size_t step = 2 * jslot_bytes(R);
+  for (int t = t0; t < jtri(R) + R; t += n) {
+    if (t < jtri(R)) {
+      int ti = 0;
+      while (jtri(ti + 1) <= t) ++ti;
+      double a = (double)reinterpret_cast<const float*>(p0)[t];
+#pragma unroll 8
+      for (int64_t k = 0; k < np; ++k) a += (double)reinterpret_cast<const float*>(pk + k * step)[t];
+      tri(ti, t - jtri(ti), a);
+    } else {
+      const int ti = t - jtri(R);
+      const size_t at = jslot_bytes(R) - sizeof(double) * (R - ti);
+      double a = *reinterpret_cast<const double*>(p0 + at);
+#pragma unroll 8
+      for (int64_t k = 0; k < np; ++k) a += *reinterpret_cast<const double*>(pk + k * step + at);
+      rhs(ti, a);
+    }
+  }
+}
+
 // The systems of 32 rows and their solutions.  Shared memory: the lower
 // triangles [entry][row] and right sides [column][row] in FP64 (rows padded to
 // kJTileLd: conflict-free by entry and by row), and a staging tile per warp.
@@ -317,29 +346,9 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
         const int rr = __ffs(heavy) - 1;
         const int64_t row = tile + rr * ntiles;
         const int64_t b = yptr[row], e = yptr[row + 1];
-        // the row's pieces in order, a thread per entry
-        const int64_t k0 = b / kHeavyRatings, k1 = (e - 1) / kHeavyRatings;
-        const unsigned char* p0 = slots + (2 * k0 + (b % kHeavyRatings ? 1 : 0)) * jslot_bytes(R);
-        const unsigned char* pk = slots + 2 * (k0 + 1) * jslot_bytes(R);  // the pieces after the first
-        const int64_t np = k1 - k0;
-        const size_t step = 2 * jslot_bytes(R);
-        for (int t = threadIdx.x; t < jtri(R) + R; t += kJSolveWarps * 32) {
-          if (t < jtri(R)) {
-            int ti = 0;
-            while (jtri(ti + 1) <= t) ++ti;
-            double a = (double)reinterpret_cast<const float*>(p0)[t];
-#pragma unroll 8
-            for (int64_t k = 0; k < np; ++k) a += (double)reinterpret_cast<const float*>(pk + k * step)[t];
-            Hs[t * kJTileLd + rr] = base[ti * R + (t - jtri(ti))] + a;
-          } else {
-            const int i2 = t - jtri(R);
-            const size_t at = jslot_bytes(R) - sizeof(double) * (R - i2);
-            double a = mu * (double)N[row * R + i2] + *reinterpret_cast<const double*>(p0 + at);
-#pragma unroll 8
-            for (int64_t k = 0; k < np; ++k) a += *reinterpret_cast<const double*>(pk + k * step + at);
-            xs[i2 * kJTileLd + rr] = a;
-          }
-        }
+        add_pieces(slots, b, e, R, threadIdx.x, kJSolveWarps * 32,
+                   [&](int ti, int tj, double a) { Hs[(jtri(ti) + tj) * kJTileLd + rr] = base[ti * R + tj] + a; },
+                   [&](int ti, double a) { xs[ti * kJTileLd + rr] = mu * (double)N[row * R + ti] + a; });
       }
     }
     __syncthreads();
@@ -402,6 +411,95 @@ __global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve(
     __syncthreads();  // before the next 32 rows
   }
 }
+
+// The same for a side of few rows: a warp per row, lane m on row m of its system
+// (R <= 32).  An FP64 instruction serves one row here, but the chain of a row is
+// R^2 / 2 of them, not R^3 / 6, which is what counts where the SMs have a block or
+// less each.
+template <typename T, int RP>
+__global__ void __launch_bounds__(kJSolveWarps * 32) joint_solve_few(
+    const int64_t* __restrict__ yptr, const int32_t* __restrict__ ycol,
+    const float* __restrict__ yval, const T* __restrict__ other, const float* __restrict__ N,
+    const double* __restrict__ base, double mu, int64_t rows, int R,
+    const unsigned char* __restrict__ slots, T* __restrict__ F, int32_t* __restrict__ bad_flag) {
+  using S = JShape<RP>;
+  extern __shared__ __align__(16) double jsm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane % RP, h = lane / RP;
+  const int LD = R + 1, own = R * LD + R;
+  // per warp: the lower triangle [R][LD] and the right side [R]; then the tiles
+  double* H = jsm + (size_t)warp * own;
+  double* x = H + (size_t)R * LD;
+  float* tile = reinterpret_cast<float*>(jsm + ((size_t)kJSolveWarps * own + 1) / 2 * 2) + (size_t)warp * 32 * S::LD;
+  const int64_t row0 = (int64_t)blockIdx.x * kJSolveWarps, row = row0 + warp;
+  if (row < rows) {
+    const int64_t b = yptr ? yptr[row] : 0, e = yptr ? yptr[row + 1] : 0;
+    if (e - b <= kHeavyRatings) {
+      float hrow[S::CPL];
+      double rhs;
+      joint_accumulate<T, RP>(ycol, yval, other, b, e, R, tile, hrow, rhs);
+#pragma unroll
+      for (int c = 0; c < S::CPL; ++c) {
+        const int j = h * S::CPL + c;
+        if (i < R && j <= i) H[i * LD + j] = base[i * R + j] + (double)hrow[c];
+      }
+      if (h == 0 && i < R) x[i] = mu * (double)N[row * R + i] + rhs;
+    }
+  }
+  if (slots && yptr) {  // heavy rows, by the whole block
+    for (int w = 0; w < kJSolveWarps && row0 + w < rows; ++w) {
+      const int64_t r = row0 + w, b = yptr[r], e = yptr[r + 1];
+      if (e - b <= kHeavyRatings) continue;
+      double* Hw = jsm + (size_t)w * own;
+      add_pieces(slots, b, e, R, threadIdx.x, kJSolveWarps * 32,
+                 [&](int ti, int tj, double a) { Hw[ti * LD + tj] = base[ti * R + tj] + a; },
+                 [&](int ti, double a) { Hw[R * LD + ti] = mu * (double)N[r * R + ti] + a; });
+    }
+    __syncthreads();
+  }
+  __syncwarp();
+  if (row >= rows) return;
+  bool bad = false;
+  double xl = lane < R ? x[lane] : 0.0, inv_own = 0.0;
+  for (int k = 0; k < R; ++k) {  // column k of L below the diagonal, then L y = rhs as it goes
+    const double d = H[k * LD + k];
+    bad |= !(d > 0.0);
+    const double inv = rsqrt(fmax(d, 1e-300));
+    double lk = 0.0;
+    if (lane > k && lane < R) {
+      lk = H[lane * LD + k] * inv;
+      H[lane * LD + k] = lk;
+    }
+    if (lane == k) inv_own = inv;
+    const double yk = __shfl_sync(kFull, xl, k) * inv;
+    if (lane == k) xl = yk;
+    else if (lane > k) xl -= lk * yk;
+    __syncwarp();
+    if (lane > k && lane < R)
+      for (int m = k + 1; m <= lane; ++m) H[lane * LD + m] -= lk * H[m * LD + k];
+    __syncwarp();
+  }
+  for (int k = R - 1; k >= 0; --k) {  // L^T x = y
+    const double xk = __shfl_sync(kFull, xl * inv_own, k);
+    if (lane == k) xl = xk;
+    else if (lane < k) xl -= H[k * LD + lane] * xk;
+  }
+  if (lane < R) st_elem(F + row * R + lane, (float)xl);
+  if (bad && lane == 0) atomicOr(bad_flag, 1);
+}
+
+template <int RP>
+size_t joint_few_smem(int R) {
+  return sizeof(double) * (((size_t)kJSolveWarps * (R * (R + 1) + R) + 1) / 2 * 2) +
+         sizeof(float) * kJSolveWarps * 32 * JShape<RP>::LD;
+}
+
+// Which row solver: a warp per row while that is at most a block per SM, and above
+// R = 28, where joint_solve's systems leave room for one block per SM.  A sweep
+// with 8 ratings per row, warp per row against 32 rows per block: 1,000 rows per
+// side 304 and 413 us at R = 16, 397 and 750 at R = 24 (a warp per row without
+// these kernels 577 and 717); 2,500 rows 461 and 420, 763 and 752; 50,000 rows
+// 3.54 and 1.17 ms at R = 16, 8.35 and 8.36 at R = 28, 9.86 and 11.46 at R = 32.
+bool few_rows(int64_t rows, int R) { return rows <= 152 * kJSolveWarps || R > 28; }
 
 template <int RP>
 size_t joint_solve_smem(int R) {
@@ -616,9 +714,12 @@ dfacto_status joint_solve_side(dfacto_t* h, int side) {
         J->ptr[side], J->col[side], J->val[side], other, rows, J->nnzY, R, J->slots);
     DF_COUNT();
   }
-  const size_t smem = joint_solve_smem<RP>(R);
-  DF_CUDA(h, ensure_dynamic_smem(reinterpret_cast<const void*>(joint_solve<T, RP>), smem));
-  joint_solve<T, RP><<<jgrid(rows, 32), kJSolveWarps * 32, smem, s>>>(
+  const bool few = few_rows(rows, R);
+  const size_t smem = few ? joint_few_smem<RP>(R) : joint_solve_smem<RP>(R);
+  const unsigned grid = few ? (unsigned)((rows + kJSolveWarps - 1) / kJSolveWarps) : jgrid(rows, 32);
+  auto kernel = few ? joint_solve_few<T, RP> : joint_solve<T, RP>;
+  DF_CUDA(h, ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem));
+  kernel<<<grid, kJSolveWarps * 32, smem, s>>>(
       rated ? J->ptr[side] : nullptr, rated ? J->col[side] : nullptr, rated ? J->val[side] : nullptr,
       other, h->N, J->base, J->mu, rows, R, J->slots, static_cast<T*>(h->F[side]),
       h->flags + kFlagInternal);
