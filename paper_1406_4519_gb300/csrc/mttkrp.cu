@@ -229,7 +229,6 @@ int walk_segment(int dtype, int seg_opt) {
 }
 
 WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, int vec_opt) {
-  (void)nfib;
   WalkCfg c;
   // Default: one 16-byte load per lane and factor row (4 FP32 or 8 BF16
   // columns), measured fastest on the 50M-nonzero power-law workload at
@@ -249,12 +248,16 @@ WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, in
   // kWalkWaves times over (27,773 nonzeros, R = 24: 57 us for three modes with
   // 32, 108 with 128).  Never longer: a segment is the longest FP32 chain of a
   // row's sum (50M power-law nonzeros, R = 32: 860 us per mode with 256 and 901
-  // with 128, but 2.2e-7 from 64 bits and 1.8e-7).
+  // with 128, but 2.2e-7 from 64 bits and 1.8e-7).  Where fibers hold sixteen
+  // nonzeros or more there is less to wait for within a segment and one wave is
+  // enough (300 x 200 x 100, R = 16: 2M nonzeros 110 us with 32, 92 with 64; 4M
+  // 155 with 64, 135 with 128; the walk before this one took 104 and 150).
   const int segs = kWalkWarps * (32 / G);
   int seg = seg_opt;
   if (seg <= 0) {
     seg = 128;
-    while (seg > 32 && nnz < (int64_t)segs * seg * kWalkWaves * 152 * 2) seg >>= 1;
+    const int waves = nnz >= 16 * nfib ? 1 : kWalkWaves;
+    while (seg > 32 && nnz < (int64_t)segs * seg * waves * 152 * 2) seg >>= 1;
   }
   seg = std::max(32, (seg + 31) / 32 * 32);
   c.seg = seg;

@@ -61,3 +61,12 @@ def test_default_segments_hold_no_longer_chain_than_128():
         t.set_factors(F)
         got.append([t.mttkrp(m) for m in range(3)])
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+def test_segments_are_not_cut_short_where_fibers_are_long():
+    # 66 to 200 nonzeros per fiber: one wave of CTAs is enough
+    dims = [300, 200, 100]
+    for nnz, R, seg in ((2000000, 16, 64), (4000000, 16, 128)):
+        idx, val = synth.uniform_tensor(dims, nnz, seed=5, device="cuda")
+        t = dfacto.Tensor(idx, val, dims, rank=R)
+        assert list(dfacto.dfacto_get_info(t.h).seg_nnz) == [seg] * 3
