@@ -11,11 +11,6 @@ namespace {
 
 constexpr int kFixThreads = 256;
 constexpr int kFixWarps = kFixThreads / 32;
-// Waves of walk CTAs (152 SMs, two resident) below which segments get shorter.
-// Two, against one and four: 121, 124 and 121 us per mode of 5M uniform nonzeros
-// at R = 4 (segments of 32, 64, 32), 114, 114 and 112 at R = 16 (128, 128, 64);
-// eight other sizes of 10,000 to 5M nonzeros within 3%.
-constexpr int kWalkWaves = 2;
 constexpr int kAheadCols = 32;  // carry values per lane a warp loads before adding them
 
 // One block per CTA c (grid-stride): if c's last partial run belongs to a row r
@@ -244,20 +239,21 @@ WalkCfg choose_walk(int R, int dtype, int64_t nnz, int64_t nfib, int seg_opt, in
   c.G = G;
   c.kernel = 2;  // fiber ends from the end bitmask (faster on every measured shape)
 
-  // Segment length: 128, or shorter where the CTAs would not fill the GPU
-  // kWalkWaves times over (27,773 nonzeros, R = 24: 57 us for three modes with
-  // 32, 108 with 128).  Never longer: a segment is the longest FP32 chain of a
-  // row's sum (50M power-law nonzeros, R = 32: 860 us per mode with 256 and 901
-  // with 128, but 2.2e-7 from 64 bits and 1.8e-7).  Where fibers hold sixteen
-  // nonzeros or more there is less to wait for within a segment and one wave is
-  // enough (300 x 200 x 100, R = 16: 2M nonzeros 110 us with 32, 92 with 64; 4M
-  // 155 with 64, 135 with 128; the walk before this one took 104 and 150).
+  // Segment length: 128, or shorter where that leaves SMs without work: fewer
+  // than a CTA per SM, or, with eight lanes per group and short fibers, than
+  // four (such CTAs wait most and three are resident).  Never longer: a segment is
+  // the longest FP32 chain of a row's sum (50M power-law nonzeros, R = 32: 860 us
+  // per mode with 256 and 901 with 128, but 2.2e-7 from 64 bits and 1.8e-7).
+  // Three modes with segments of 32, 64 and 128: uniform nonzeros 1M, R = 4: 103,
+  // 146, 225 us; 8M, R = 4: 538, 463, 429; 2M, R = 16: 182, 147, 130; 2M in fibers
+  // of 66, R = 16: 110, 92, 80; power-law nonzeros 2M, R = 32: 193, 178, 208.  Walk
+  // 1 falls behind further with short ones (8M, R = 1: 1,569, 780, 755).
   const int segs = kWalkWarps * (32 / G);
   int seg = seg_opt;
   if (seg <= 0) {
     seg = 128;
-    const int waves = nnz >= 16 * nfib ? 1 : kWalkWaves;
-    while (seg > 32 && nnz < (int64_t)segs * seg * waves * 152 * 2) seg >>= 1;
+    const int64_t ctas = 152 * (G >= 8 && nnz < 16 * nfib ? 4 : 1);
+    while (seg > 32 && nnz < (int64_t)segs * seg * ctas) seg >>= 1;
   }
   seg = std::max(32, (seg + 31) / 32 * 32);
   c.seg = seg;

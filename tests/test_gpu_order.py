@@ -63,10 +63,13 @@ def test_default_segments_hold_no_longer_chain_than_128():
     assert all(torch.equal(a, b) for a, b in zip(*got))
 
 
-def test_segments_are_not_cut_short_where_fibers_are_long():
-    # 66 to 200 nonzeros per fiber: one wave of CTAs is enough
-    dims = [300, 200, 100]
-    for nnz, R, seg in ((2000000, 16, 64), (4000000, 16, 128)):
+def test_segments_are_not_cut_short_where_the_sms_have_work():
+    # (dims, nonzeros, rank, walk) -> segment length: fibers of 66 to 200 nonzeros,
+    # and one lane per segment, where short segments made walk 1 half as fast
+    for dims, nnz, R, seg in (([300, 200, 100], 2000000, 16, 128), ([300, 200, 100], 4000000, 32, 128),
+                              ([300000, 200000, 100000], 8000000, 1, 128),
+                              ([300000, 200000, 100000], 8000000, 4, 128)):
         idx, val = synth.uniform_tensor(dims, nnz, seed=5, device="cuda")
-        t = dfacto.Tensor(idx, val, dims, rank=R)
-        assert list(dfacto.dfacto_get_info(t.h).seg_nnz) == [seg] * 3
+        for walk in (1, 2):
+            t = dfacto.Tensor(idx, val, dims, rank=R, walk=walk)
+            assert list(dfacto.dfacto_get_info(t.h).seg_nnz) == [seg] * 3
