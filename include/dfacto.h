@@ -78,8 +78,9 @@ typedef enum dfacto_dtype {
  *                 is the same sums up to their order), which the handle
  *                 allocates on first use.
  *   walk          MTTKRP kernel: 1 detects fiber ends from the fiber pointers
- *                 as it walks, 2 from a per-nonzero end bitmask and closes the
- *                 fibers of a few steps together; 0 lets the library choose.
+ *                 as it walks, 2 from a per-nonzero end bitmask, gathering the
+ *                 rows of both factors for a few steps together; 0 lets the
+ *                 library choose.
  *                 Other values are refused (DFACTO_EINVAL).  Both compute the
  *                 same sums in the same order.
  *   line_search   GD step size (dfacto_gd_iter): 0 (default) backtracking from
@@ -402,7 +403,9 @@ typedef struct {
   int32_t reserved[6];  /* zero */
 } dfacto_batch_options;
 
-/* Defaults: graph on, autotune on. */
+/* Defaults: graph on, autotune on.  Rank classes with BF16 factors have one walk
+ * shape per rank, whatever the times, so that their results do not depend on
+ * timing: BF16 storage turns a last bit of a sum into 2^-9 of a factor entry. */
 void dfacto_batch_options_init(dfacto_batch_options* opt);
 
 /*

@@ -567,8 +567,10 @@ cudaError_t radix_pass(const uint64_t* ki, const uint32_t* vi, uint64_t* ko, uin
 // Digit passes for an nbits-wide range of n keys: of 8 or 9 bits, whichever is
 // the cheaper.  A nine-bit pass over 50M pairs costs 1.23 times an eight-bit one
 // (534 against 434 us: twice the digits, so half the run each tile writes of
-// one), over 500,000 pairs 1.05 times (23 against 22 us).  Returns the cost in
-// eight-bit passes.
+// one), over 500,000 pairs 1.05 times (23 against 22 us).  Builds with 54-bit keys
+// sorted by six nine-bit digits and by seven eight-bit ones: 532 and 544 us at
+// 500,000 pairs, 1,114 and 1,122 at 4M, 1,817 and 1,809 at 8M, 5,800 and 5,753 at
+// 32M, so the line lies between 4M and 8M.  Returns the cost in eight-bit passes.
 double radix_plan(int nbits, int64_t n, int* passes, int* bits) {
   const double w9 = n > (int64_t)1 << 22 ? 1.23 : 1.05;
   const int p8 = nbits > 0 ? (nbits + 7) / 8 : 0, p9 = nbits > 0 ? (nbits + 8) / 9 : 0;

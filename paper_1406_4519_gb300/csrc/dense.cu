@@ -1147,23 +1147,6 @@ int pass_blocks(int64_t rows) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, kPassWave));
 }
 
-// Row r of N (R columns) zero-padded to RT.
-template <int RT>
-__device__ __forceinline__ void load_row(const float* __restrict__ N, int64_t r, int R, float (&n)[RT]) {
-  const float* p = N + r * R;
-  if ((R & 3) == 0) {
-#pragma unroll
-    for (int c4 = 0; c4 < RT / 4; ++c4) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (4 * c4 < R) v = __ldg(reinterpret_cast<const float4*>(p) + c4);
-      n[4 * c4] = v.x; n[4 * c4 + 1] = v.y; n[4 * c4 + 2] = v.z; n[4 * c4 + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < RT; ++c) n[c] = c < R ? __ldg(p + c) : 0.f;
-  }
-}
-
 // Columns [c0, c0 + CW) of o = n W (W: RT x RT in shared memory, row k holds
 // the coefficients of n[k]); k ascends, so every caller gets the same values.
 template <int RT, int CW>
@@ -1696,7 +1679,8 @@ __device__ __forceinline__ void store_gram_partial(const float (&a32)[16], float
 // Pass 1: colsq[vb][c] = sum over the block's rows of (N W)[row, c]^2.  A tile
 // of kT rows is loaded into shared memory with coalesced loads; thread t then
 // takes row t of the tile.  Each thread sums its rows in FP32; the block adds
-// the threads in FP64, in thread order.
+// the threads in FP64: sixteen threads in order per part, then the sixteen parts
+// in order.
 template <int RT>
 __device__ __forceinline__ void colnorm_rows_body(const float* __restrict__ N, int ldN,
                                                   const float* __restrict__ W32, int64_t rows, int R,

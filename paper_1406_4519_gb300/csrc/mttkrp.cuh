@@ -397,17 +397,17 @@ __global__ void __launch_bounds__(kWalkWarps * 32) mttkrp_walk(const MttkrpParam
 //
 // What bounds it: the latency of the gathers against the registers that hold
 // them.  The gathers mostly hit L1 and L2 (a bare probe of 128-byte rows reaches
-// 140 G rows/s from L2 on this GPU, the walk 80 on 50M power-law nonzeros at
+// 140 G rows/s from L2 on this GPU, the walk 75 on 50M power-law nonzeros at
 // R = 32), so what counts is how many are in flight and how few instructions
 // stand between two rounds: the earlier form of this walk parked the fiber sums
 // in shared memory and folded them in a second, dependent round of loads (18
 // warp instructions per nonzero, now 8).  Per mode of 50M power-law nonzeros,
-// before and now: R = 32 1.05 and 0.85 ms, R = 16 0.64 and 0.52, R = 8 0.59 and
-// 0.40, R = 32 with BF16 factors 1.04 and 0.56.  Slower here: the streams
-// staged in shared memory by cp.async (0.87 ms at R = 32, 12 instructions), the
-// sum taken term by term without fibers (0.80 ms at R = 32 but 1.1 times slower
-// at R = 12 to 16, and a gather more per nonzero), and eight FP32 columns per
-// lane.
+// before and now: R = 32 1.05 and 0.90 ms, R = 16 0.64 and 0.55, R = 8 0.59 and
+// 0.40, R = 32 with BF16 factors 1.04 and 0.58.  Slower, all with segments of 256
+// where this walk takes 0.86 ms at R = 32: the streams staged in shared memory by
+// cp.async (0.87 ms, 12 instructions), the sum taken term by term without fibers
+// (0.80 ms at R = 32 but 1.1 times slower at R = 12 to 16, and a gather more per
+// nonzero), and eight FP32 columns per lane.
 //
 // nz_idx, nz_val and the bit words are allocated up to a multiple of 32
 // nonzeros, zero past nnz: those positions read row 0, and as they end no
