@@ -174,8 +174,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32) dual_walk(const DualParams a)
 //
 // Bound by the latency of its gathers against the registers that hold them, like
 // mttkrp_walk2.  50M power-law nonzeros, R = 32: 2.30 ms with the fiber sums
-// parked in shared memory and folded after a second round of loads, 1.97 now;
-// R = 10 (padded to 12): a GD step 4.59 -> 3.29 ms with the walks and row passes.
+// parked in shared memory and folded after a second round of loads, 1.98 now;
+// R = 10 (padded to 12): a GD step 4.54 -> 3.26 ms with the walks and row passes.
 // ---------------------------------------------------------------------------
 // Positions gathered together, at most (two: 128 registers, two CTAs per SM,
 // without spills; four spill and take 5% longer, two at 80 registers 20%).
