@@ -338,8 +338,8 @@ dfacto_status time_class(dfacto_batch* b, int k, int reps, double* ms) {
 // A BF16 class has one: its shape sets the order of its sums, and BF16 storage
 // turns a last bit of a sum into 2^-9 of a factor entry now and then, so a shape
 // chosen by time would make the factors of a batch differ between two creations.
-// Segments of 64 with four columns per lane (eight where four would take more
-// than four lanes) are what timing mostly chose when every BF16 class was timed;
+// Segments of 64 with four columns per lane (eight at R = 24 and 32, where four
+// would take eight lanes) are what timing mostly chose when every BF16 class was timed;
 // ranks without such a shape keep the default.  48 uneven jobs, ranks 8, 16, 32
 // (32M nonzeros): 1.59 ms for the three modes' walks, 1.49 with segments of 128.
 std::vector<WalkCfg> candidates(const BatchClass& C) {
